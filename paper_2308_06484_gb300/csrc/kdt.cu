@@ -22,6 +22,7 @@
 
 #include "../../include/kdt.h"
 #include "kdt_kernels.cuh"
+#include "kdt_rounds.cuh"
 #include "kdt_dcalc.cuh"
 #include "kdt_plan.cuh"
 #include "kdt_tc.cuh"
@@ -87,6 +88,10 @@ struct kdt {
     // build / export temporaries (kept between calls)
     Buf key, bord, hist, hoff, exp_cnt, exp_off, exp_fill, exp_out;
     Buf btab, blev;  // batched build: per-instance tables, per-level item offsets
+    // rounds (kdt_rounds.cuh): of a build, and of the steps (sized for mcap moves)
+    Buf rb_cnt, rb_lost, rb_hdr, rb_rec, rb_queue, rb_left;
+    Buf rm_cnt, rm_lost, rm_hdr, rm_rec, rm_slots, rm_left;
+    int rm_rounds = 0, rm_ops = 0;
     // d-calculation: neighbour lists, results, running minimum (per N)
     Buf nb_deg, nb_off, nb_list, dc_dist, dc_cmin, dc_scal;
     int64_t d2_run = INT64_MAX;
@@ -128,7 +133,7 @@ struct kdt {
     int tune_count = 0;
     double tune_ms[9] = {0};
     // host side
-    int *hscal = nullptr;  // pinned copy of the scalars
+    int *hscal = nullptr;  // pinned copy of the scalars (and two words more)
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr, ev3 = nullptr;
     kdt_stats stats{};
     // learned locate proposal and its training rows (kdt_mlp.cuh)
@@ -279,6 +284,7 @@ Inst make_inst(kdt *h)
     I.qhist = h->qhist;
     I.stride = h->cfg.partition_order == 0 && !h->qhist ? h->stride : 1;
     I.ncells_dyn = h->qhist ? h->scal + S_NCELLS : nullptr;
+    I.pending = nullptr;
     return I;
 }
 
@@ -389,9 +395,145 @@ int certify_and_repair(kdt *h, bool full, int s0, int nslots, int wraps, int *de
     return 0;
 }
 
+// the counters of `rounds` rounds in one buffer: heads, offsets and losers (rounds + 1
+// entries each), the left list's length, the moves pending; `ops` operations a round
+size_t round_counter_ints(int rounds) { return 3 * (size_t)(rounds + 1) + 2; }
+
+Rounds make_rounds(const Buf &cnt, int rounds, const Buf &lost, const Buf &hdr, const Buf &rec, int ops)
+{
+    Rounds R;
+    int *c = (int *)cnt.p;
+    R.head = c;
+    R.off = c + (rounds + 1);
+    R.lostcnt = c + 2 * (rounds + 1);
+    R.left_count = c + 3 * (rounds + 1);
+    R.pending = R.left_count + 1;
+    R.lost[0] = (int *)lost.p;
+    R.lost[1] = (int *)lost.p + ops;
+    R.hdr = (int4 *)hdr.p;
+    R.rec = (int4 *)rec.p;
+    R.slots = nullptr;
+    R.left = nullptr;
+    R.div = 0;
+    R.few = 0;
+    R.base = 0;
+    R.ops = ops;
+    return R;
+}
+
+// A round's kernels for at most `most` operations; wide: 32 lanes plan an operation (twice
+// the limits of 16 lanes, half the rate); last: what the plan cannot take is left out.
+template <bool MOVE>
+void launch_round(kdt *h, cudaStream_t st, const Dev &d, const Rounds &R, int b, long long most, const RoundMoves &M,
+                  const RoundBuild &B, bool wide, bool last)
+{
+    const int sms = sm_count(h->device);
+    // (a warp for every operation, while the GPU has room for that many)
+    const long long pb = std::min<long long>((most * 32 + ROUND_THREADS - 1) / ROUND_THREADS, 32ll * sms);
+    auto plan = wide ? k_round_plan<MOVE, 32> : k_round_plan<MOVE, 16>;
+    plan<<<(int)std::max(1ll, pb), ROUND_THREADS, 0, st>>>(d, R, b, M, B, last ? 1 : 0);
+    const long long cb = std::min<long long>((most * ROUND_LANES + 255) / 256, 8ll * sms);
+    k_round_commit<MOVE><<<(int)std::max(1ll, cb), 256, 0, st>>>(d, R, b, M, B);
+}
+
+// A round of a build takes up to one BUILD_DIV-th as many new points as are in, or as many as
+// are in while those are at most BUILD_FEW: the more, the more of them meet (a sixteenth:
+// 1.3 attempts per insertion, an eighth: 1.7, a quarter: 2.8, all: 8.8; counted on 2e5
+// uniform points), the fewer, the more rounds.  Small rounds cost their latency only,
+// large ones their attempts.  1e6 points: 4 / 0 20.4 ms, 8 / 0 10.8, 12 / 0 9.8, 12 / 2048 9.7,
+// 12 / 8192 11.5, 16 / 4096 9.9 against 10.3 with 12 / 4096.
+constexpr int BUILD_DIV = 12, BUILD_FEW = 2048;
+
+// Insert every point of the instances whose first triangles are in (the points in Hilbert
+// order, the instances' levels in lv: ni + 1 item offsets per level, on the device at
+// dlv) in rounds, then what the rounds left with one warp per point.  Slots s0 ..
+// s0 + nslots - 1 are the instances'.  Returns an ABI code.
+int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const int *dlv, int levels, int s0,
+                  int nslots)
+{
+    cudaStream_t st = h->stream;
+    const int ni = B.ninst;
+    long long total = 0;
+    for (int l = 0; l < levels; ++l) total += lv[(size_t)l * (ni + 1) + ni];
+    const long long np = total + ni;
+    const int ops = (int)std::min<long long>(ROUND_OPS, std::max<long long>(64, std::max<long long>(np / BUILD_DIV, std::min<long long>(np, BUILD_FEW)) + 64));
+    if (grow(h->rb_cnt, round_counter_ints(ROUND_MAX) * sizeof(int)) || grow(h->rb_lost, 2 * (size_t)ops * sizeof(int)) ||
+        grow(h->rb_hdr, (size_t)ops * sizeof(int4)) || grow(h->rb_rec, (size_t)ops * 2 * RT * sizeof(int4)) ||
+        grow(h->rb_queue, (size_t)np * sizeof(int)) ||
+        grow(h->rb_left, (size_t)np * sizeof(int)))
+        return KDT_ERR_CUDA;
+    Rounds R = make_rounds(h->rb_cnt, ROUND_MAX, h->rb_lost, h->rb_hdr, h->rb_rec, ops);
+    R.left = (int *)h->rb_left.p;
+    R.div = BUILD_DIV;
+    R.few = BUILD_FEW;
+    R.base = 3 * ni;
+    B.queue = (const int *)h->rb_queue.p;
+    B.total = (int)total;
+    CK(cudaMemsetAsync(h->rb_cnt.p, 0, round_counter_ints(ROUND_MAX) * sizeof(int), st));
+    int at = 0;
+    for (int l = levels - 1; l >= 0; --l) {
+        const int items = lv[(size_t)l * (ni + 1) + ni];
+        if (items <= 0) continue;
+        long long stride = std::max(1ll, std::llround(0.6180339887498949 * (double)items));
+        while (std::gcd(stride, (long long)items) != 1) ++stride;
+        k_build_queue<<<thread_grid(h, items, 256), 256, 0, st>>>(B, ni > 1 ? dlv + (size_t)l * (ni + 1) : h->d_pofs, l, items, (int)stride,
+                                                                 (int *)h->rb_queue.p + at);
+        h->stats.kernel_launches++;
+        at += items;
+    }
+    int b = 0;
+    const RoundMoves M{nullptr};
+    long long in = R.base;  // points in at most
+    int batch = h->cfg.build_warps > 0 ? 0 : (int)(11.0 * std::log((double)np / ni)) + 4;
+    bool wide = false;
+    for (int pending = -1; batch > 0 && b + batch <= ROUND_MAX;) {
+        for (int i = 0; i < batch; ++i, ++b) {
+            const long long most = std::min<long long>(
+                ops, std::max<long long>(64, std::max<long long>(in / BUILD_DIV, std::min<long long>(in, BUILD_FEW))));
+            launch_round<false>(h, st, d, R, b, most, M, B, wide, false);
+            in = std::min(in + most, np);
+        }
+        h->stats.kernel_launches += 2 * batch;
+        CK(cudaGetLastError());
+        int *hs = h->hscal + S_NUM;  // pinned
+        CK(cudaMemcpyAsync(hs, R.head + b, sizeof(int), cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(hs + 1, R.lostcnt + b, sizeof(int), cudaMemcpyDeviceToHost, st));
+        if (sync_scalars(h)) return KDT_ERR_CUDA;
+        if (h->hscal[S_STATUS]) return dev_to_abi(h->hscal[S_STATUS]);
+        const int now = B.total - hs[0] + hs[1];
+        if (now == 0 || (wide && now == pending)) break;
+        // the rest in 32 lanes once it is small (what 16 cannot take is among it)
+        wide = wide || (hs[0] == B.total && now <= 4096);
+        pending = now;
+        batch = 8;
+    }
+    k_clear_owner<<<thread_grid(h, nslots, 256), 256, 0, st>>>(d.tn, s0, nslots);
+    k_build_rest<<<thread_grid(h, total, 256), 256, 0, st>>>(R, b, B);
+    h->stats.kernel_launches += 2;
+    CK(cudaMemcpyAsync(h->hscal + S_NUM, R.left_count, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    const int left = h->hscal[S_NUM];
+    if (left > 0) {
+        // about 16 triangles of room per concurrent insertion: more warps than that only
+        // collide on the same cavities (claims fail, back off, retry)
+        long long warps = std::min<long long>(left, std::max<long long>(8ll * ni, (np - left) / 8));
+        if (h->cfg.build_warps > 0) warps = h->cfg.build_warps;
+        int blocks = warp_grid(h, warps, 64), threads = WPB * 32;
+        if (h->cfg.build_warps > 0 && h->cfg.build_warps < WPB) {
+            blocks = 1;
+            threads = 32 * h->cfg.build_warps;
+        }
+        k_insert_left<<<blocks, threads, 0, st>>>(d, R.left, left, B);
+        h->stats.kernel_launches++;
+        CK(cudaGetLastError());
+    }
+    if (sync_scalars(h)) return KDT_ERR_CUDA;
+    return h->hscal[S_STATUS] ? dev_to_abi(h->hscal[S_STATUS]) : KDT_OK;
+}
+
 // Build the triangulation of instance i from the positions in h->xy: Hilbert order
-// over a grid on its bounding box, the first non-degenerate triangle, then parallel
-// insertion level by level (positions (2j+1) * 2^level walk from position 2j * 2^level),
+// over a grid on its bounding box, the first non-degenerate triangle, then rounds of
+// insertions level by level (positions (2j+1) * 2^level walk from position 2j * 2^level),
 // then certification and repair.  Returns an ABI code.
 int rebuild_instance(kdt *h, int i)
 {
@@ -440,29 +582,12 @@ int rebuild_instance(kdt *h, int i)
     h->stats.kernel_launches++;
     int K = 0;
     while ((1ll << (K + 1)) < (long long)n) ++K;
-    long long inserted = 3;
-    for (int lev = K; lev >= 0; --lev) {
-        long long items = ((long long)n - 1 + (1ll << lev)) >> (lev + 1);  // odd multiples of 2^lev below n
-        if (items <= 0) continue;
-        // about 16 triangles of room per concurrent insertion: more warps than that only
-        // collide on the same cavities (claims fail, back off, retry)
-        long long conc = inserted / 8;
-        if (conc < 8) conc = 8;
-        if (h->cfg.build_warps > 0) conc = h->cfg.build_warps;
-        long long warps = items < conc ? items : conc;
-        int blocks = warp_grid(h, warps, 64), threads = WPB * 32;
-        if (h->cfg.build_warps > 0 && h->cfg.build_warps < WPB) {
-            blocks = 1;
-            threads = 32 * h->cfg.build_warps;
-        }
-        k_insert_level<<<blocks, threads, 0, st>>>(d, order, lev, (int)items, h->scal + S_TRIS, n, s0 + capi);
-        h->stats.kernel_launches++;
-        CK(cudaGetLastError());
-        inserted += items;
-    }
-    if (sync_scalars(h)) return KDT_ERR_CUDA;
-    if (h->hscal[S_STATUS]) return dev_to_abi(h->hscal[S_STATUS]);
-    if (h->hscal[S_TRIS] != s0 + capi) return KDT_ERR_INTERNAL;
+    std::vector<int> lv(2 * (size_t)(K + 1), 0);
+    for (int lev = 0; lev <= K; ++lev) lv[2 * lev + 1] = (int)(((long long)n - 1 + (1ll << lev)) >> (lev + 1));
+    // (the order holds this instance alone: its positions start at d_pofs[0] = 0; with one
+    // instance no level's offsets are searched, so the same zero stands for each)
+    RoundBuild B{nullptr, order, h->scal + S_THIRD, h->d_pofs, h->d_tofs + i, 1, 0, n};
+    if (const int rc = insert_rounds(h, d, B, lv, nullptr, K + 1, s0, capi)) return rc;
     int ds = 0;
     if (certify_and_repair(h, true, s0, capi, 1, &ds)) return KDT_ERR_CUDA;
     if (ds) return dev_to_abi(ds);
@@ -559,29 +684,8 @@ int rebuild_batch(kdt *h)
     }
     if (grow(h->blev, lv.size() * sizeof(int))) return KDT_ERR_CUDA;
     CK(cudaMemcpyAsync(h->blev.p, lv.data(), lv.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-    std::vector<long long> inserted(ni, 3);
-    for (int lev = Kmax; lev >= 0; --lev) {
-        const int *o = lv.data() + (size_t)lev * (ni + 1);
-        const int items = o[ni];
-        if (items <= 0) continue;
-        // about 16 triangles of room per concurrent insertion in every instance
-        long long conc = 0;
-        for (int i = 0; i < ni; ++i)
-            if (o[i + 1] > o[i]) conc += std::max(8ll, inserted[i] / 8);
-        if (h->cfg.build_warps > 0) conc = h->cfg.build_warps;
-        long long warps = std::min<long long>(items, conc);
-        k_insert_level_batch<<<warp_grid(h, warps, 64), WPB * 32, 0, st>>>(
-            d, order, lev, items, (const int *)h->blev.p + (size_t)lev * (ni + 1), h->d_pofs, h->d_tofs, ni, tcount);
-        h->stats.kernel_launches++;
-        CK(cudaGetLastError());
-        for (int i = 0; i < ni; ++i) inserted[i] += o[i + 1] - o[i];
-    }
-    std::vector<int> tc(ni);
-    CK(cudaMemcpyAsync(tc.data(), tcount, ni * sizeof(int), cudaMemcpyDeviceToHost, st));
-    if (sync_scalars(h)) return KDT_ERR_CUDA;
-    if (h->hscal[S_STATUS]) return dev_to_abi(h->hscal[S_STATUS]);
-    for (int i = 0; i < ni; ++i)
-        if (tc[i] != h->tofs[i + 1]) return KDT_ERR_INTERNAL;
+    RoundBuild B{nullptr, order, third, h->d_pofs, h->d_tofs, ni, 0, ni > 1 ? 0 : n};
+    if (const int rc = insert_rounds(h, d, B, lv, (const int *)h->blev.p, Kmax + 1, 0, h->cap)) return rc;
     int ds = 0;
     if (certify_and_repair(h, true, 0, h->cap, ni, &ds)) return KDT_ERR_CUDA;
     if (ds) return dev_to_abi(ds);
@@ -619,6 +723,38 @@ int ensure_moves(kdt *h, int64_t m)
     if (dc > (1ll << 30)) dc = 1ll << 30;
     if (dalloc(&h->dirty, (size_t)dc)) return KDT_ERR_CUDA;
     h->dirty_cap = (int)dc;
+    h->rm_rounds = 0;  // (ensure_rounds sizes them again)
+    h->gen++;
+    return 0;
+}
+
+// Rounds of a step beyond those that take every move once: the losers of the first are
+// few (one in 250 at one move per 250 uniform points, one in three where most points of
+// sparse cells move), those of the next fewer; the last ones go to the kinetic kernel.
+// An empty round costs about 5 us (4 more on 1e6 points: 85 -> 120 us a step), a round more
+// on 16e6 clustered points saves 30 us (2 rounds 1.55, 4 1.47, 6 1.43 ms), on 512 instances
+// it costs 20.
+constexpr int STEP_EXTRA_ROUNDS = 2, STEP_EXTRA_ROUNDS_MANY = 4, STEP_MANY = 32768;
+
+// Do the step's moves go through rounds?  The paper's method (delete and insert) without
+// training rows, proposal or planner; else the kinetic kernel does every move.
+bool step_in_rounds(const kdt *h)
+{
+    return h->cfg.variant == 0 && h->cfg.plan == 0 && !h->prop_on && !h->trace_x && h->cfg.kinetic_warps == 0;
+}
+
+int ensure_rounds(kdt *h)
+{
+    if (h->rm_rounds > 0) return 0;
+    const int ops = std::min(h->mcap, ROUND_OPS);
+    const int rounds =
+        (h->mcap + ops - 1) / ops + (h->mcap >= STEP_MANY ? STEP_EXTRA_ROUNDS_MANY : STEP_EXTRA_ROUNDS);
+    if (grow(h->rm_cnt, round_counter_ints(rounds) * sizeof(int)) || grow(h->rm_lost, 2 * (size_t)ops * sizeof(int)) ||
+        grow(h->rm_hdr, (size_t)ops * sizeof(int4)) || grow(h->rm_rec, (size_t)ops * 2 * RT * sizeof(int4)) ||
+        grow(h->rm_slots, (size_t)rounds * ops * RT * sizeof(int)) || grow(h->rm_left, (size_t)h->mcap * sizeof(int)))
+        return KDT_ERR_CUDA;
+    h->rm_ops = ops;
+    h->rm_rounds = rounds;
     h->gen++;
     return 0;
 }
@@ -714,9 +850,10 @@ void free_state(kdt *h)
     h->pfeat = nullptr;
     h->ppart = nullptr;
     h->qleaves = 0;
-    h->mcap = 0; h->dirty_cap = 0; h->scan_tmp_cap = 0;
+    h->mcap = 0; h->dirty_cap = 0; h->scan_tmp_cap = 0; h->rm_rounds = 0;
     Buf *bs[] = {&h->key, &h->bord, &h->hist, &h->hoff, &h->exp_cnt, &h->exp_off, &h->exp_fill, &h->exp_out,
-                 &h->btab, &h->blev,
+                 &h->btab, &h->blev, &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left,
+                 &h->rm_cnt, &h->rm_lost, &h->rm_hdr, &h->rm_rec, &h->rm_slots, &h->rm_left,
                  &h->nb_deg, &h->nb_off, &h->nb_list, &h->dc_dist, &h->dc_cmin, &h->dc_scal};
     for (Buf *b : bs) free_buf(*b);
     h->n = 0;
@@ -900,9 +1037,11 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
     // the step's control words and move offsets, from pinned host memory (a captured
     // copy reads them when the graph runs)
     CK(cudaMemcpyAsync(h->ctl, h->hctl, (4 + h->ninst + 1) * sizeof(int), cudaMemcpyHostToDevice, st));
+    const bool rounds = step_in_rounds(h);
     // scalars zero, partition lists empty, deferred entries -1: one kernel
     k_step_clear<<<thread_grid(h, std::max<long long>(h->ncells_cap, 4ll * h->mcap), 256), 256, 0, st>>>(
-        h->scal, S_NUM, h->head, h->ncells_cap, h->deferred, h->mcap);
+        h->scal, S_NUM, h->head, h->ncells_cap, h->deferred, h->mcap,
+        rounds ? (int *)h->rm_cnt.p : nullptr, rounds ? (int)round_counter_ints(h->rm_rounds) : 0);
     if (h->qhist) {
         // Fig. 4's Quad-treeDvision at the start of the step, from the points per fine
         // cell the intakes keep current: count pyramid, every fine cell's leaf, leaves
@@ -917,7 +1056,8 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
         if (scan(h, h->qflag, h->qpre, F * F, h->scal + S_NCELLS, st)) return KDT_ERR_CUDA;
         k_qt_map<<<thread_grid(h, (long long)F * F, 256), 256, 0, st>>>(h->qpre, h->qlev, D, h->qmap);
     }
-    k_intake_link<<<thread_grid(h, cap, 256), 256, 0, st>>>(d, mp, mi, I, h->cfg.domain_bits, h->head, h->next,
+    k_intake_link<<<thread_grid(h, cap, 256), 256, 0, st>>>(d, mp, mi, I, h->cfg.domain_bits,
+                                                            rounds ? nullptr : h->head, h->next,
                                                             h->old_xy, h->gmoves, h->dloc2, far2(h));
     const bool net = h->prop_on && (h->cfg.plan & PLAN_NETWORK), ordered = (h->cfg.plan & PLAN_ORDER) != 0;
     const bool tensor = net && (h->cfg.plan & PLAN_TENSOR);
@@ -950,6 +1090,19 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
     // inside a capture an event record must be an external node to keep its timestamp
     unsigned evflags = from_ctl ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (h->cfg.timing) CK(cudaEventRecordWithFlags(h->ev0, st, evflags));
+    if (rounds) {
+        Rounds R = make_rounds(h->rm_cnt, h->rm_rounds, h->rm_lost, h->rm_hdr, h->rm_rec, h->rm_ops);
+        R.slots = (int *)h->rm_slots.p;
+        R.left = (int *)h->rm_left.p;
+        const RoundMoves M{h->gmoves};
+        const RoundBuild B{nullptr, nullptr, nullptr, nullptr, nullptr, 0, mi, 0};
+        for (int b = 0; b < h->rm_rounds; ++b)
+            launch_round<true>(h, st, d, R, b, std::min(cap, h->rm_ops), M, B, b + 1 == h->rm_rounds,
+                               b + 1 == h->rm_rounds);
+        k_round_clear<<<thread_grid(h, (long long)cap * (RT / 4), 256), 256, 0, st>>>(
+            d, R, h->rm_rounds, mi, I, h->cfg.domain_bits, h->gmoves, h->old_xy, h->head, h->next);
+        I.pending = R.pending;
+    }
     int kblocks = 0, kthreads = 0;
     kinetic_shape(h, &kblocks, &kthreads);
     Dev dk = d;
@@ -1106,6 +1259,8 @@ int step_core(kdt *h, const kdt_move *moves, const int64_t *moff, int64_t m)
     if (rc) return rc;
     rc = ensure_big(h);
     if (rc) return rc;
+    if (step_in_rounds(h)) rc = ensure_rounds(h);
+    if (rc) return rc;
     if (h->qhist && h->scan_tmp_cap < (h->qF * h->qF + SCAN_TILE - 1) / SCAN_TILE + 1) {
         // the step graph scans every fine cell: its scan scratch must exist before capture
         const int c = (h->qF * h->qF + SCAN_TILE - 1) / SCAN_TILE + 1024;
@@ -1155,7 +1310,7 @@ int step_core(kdt *h, const kdt_move *moves, const int64_t *moff, int64_t m)
     h->stats.kernel_launches += 4 + ((h->cfg.plan & PLAN_ORDER) ? 2 : 0) +
                                 ((h->cfg.plan & PLAN_ORDER) || (h->prop_on && (h->cfg.plan & PLAN_NETWORK)) ? 1 : 0) +
                                 (h->prop_on && (h->cfg.plan & PLAN_NETWORK) && (h->cfg.plan & PLAN_TENSOR) ? 1 : 0) +
-                                (h->qhist ? h->qD + 5 : 0);
+                                (h->qhist ? h->qD + 5 : 0) + (step_in_rounds(h) ? 2 * h->rm_rounds + 1 : 0);
     CK(cudaStreamSynchronize(st));
     if (h->qhist) h->ncells = h->qleaves = h->hscal[S_NCELLS];
     if (timed) {
@@ -1446,7 +1601,7 @@ int kdt_create(kdt **out, const kdt_config *cfg, int device, void *cuda_stream)
     h->cfg = c;
     if (cudaMalloc(&h->scal, S_NUM * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&h->counters, C_SLOTS * sizeof(unsigned long long)) != cudaSuccess ||
-        cudaMallocHost(&h->hscal, S_NUM * sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&h->hscal, (S_NUM + 2) * sizeof(int)) != cudaSuccess ||
 
         cudaStreamCreateWithFlags(&h->cstream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreate(&h->ev0) != cudaSuccess || cudaEventCreate(&h->ev1) != cudaSuccess ||

@@ -3,7 +3,7 @@
 //   step:    k_intake_link -> k_kinetic (last warp: deferred points, certification of
 //            global-path writes) (-> k_fixup / k_certify until no violation)
 //   build:   k_range / k_bbox -> k_hilbert -> scan -> k_place_order -> k_third -> k_init
-//            -> k_insert_level (one launch per level) -> k_certify_all (-> k_fixup ...)
+//            -> rounds of insertions (kdt_rounds.cuh) -> k_certify_all (-> k_fixup ...)
 //   export:  k_exp_count -> scan -> k_exp_place -> k_exp_sortseg
 #pragma once
 #include "kdt_local.cuh"
@@ -49,6 +49,8 @@ struct Inst {
                       // it), so partitions taken at the same time lie far apart; 0 or 1:
                       // index order
     int ninst;
+    const int *pending;  // a step whose moves went through rounds: how many of them are left to
+                         // the kinetic kernel (in the partitions' lists); null: all of them
 };
 
 // Partition of a position of instance `inst`: its grid cell, or the quad-tree leaf of
@@ -283,13 +285,15 @@ __device__ __forceinline__ const int3 *step_moves(const Dev &d, const int3 *move
     return reinterpret_cast<const int3 *>(((unsigned long long)hi << 32) | lo);
 }
 
-// Start of a step: the scalars zero, every partition's move list empty, every deferred
-// entry -1 (one launch instead of three copies of memset).
-__global__ void k_step_clear(int *scal, int nscal, int *head, int ncells, int4 *deferred, int ndef)
+// Start of a step: the scalars and the rounds' counters zero, every partition's move list
+// empty, every deferred entry -1 (one launch instead of several memsets).
+__global__ void k_step_clear(int *scal, int nscal, int *head, int ncells, int4 *deferred, int ndef, int *rounds,
+                             int nrounds)
 {
     const int stride = gridDim.x * blockDim.x;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < max(ncells, ndef); i += stride) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < max(max(ncells, ndef), nrounds); i += stride) {
         if (i < nscal) scal[i] = 0;
+        if (i < nrounds) rounds[i] = 0;
         if (i < ncells) head[i] = -1;
         if (i < ndef) deferred[i] = make_int4(-1, -1, -1, -1);
     }
@@ -310,6 +314,7 @@ __device__ __forceinline__ void intake_fail(int *status, int code)
 // far2 x its partition's d_local^2 (dloc2; INT64_MAX = unknown or an empty partition)
 // is counted, and the
 // step becomes a rebuild (DEV_FAR stops the kinetic kernel before it changes anything).
+// head null: no lists (the moves go through rounds first, which link what they leave).
 __global__ void k_intake_link(Dev d, const int3 *moves, int m, Inst I, int bits, int *head, int *next,
                               int2 *old_xy, int3 *gmoves, const unsigned long long *dloc2, double far2)
 {
@@ -340,7 +345,7 @@ __global__ void k_intake_link(Dev d, const int3 *moves, int m, Inst I, int bits,
         int2 o = d.xy[g];
         old_xy[i] = o;
         gmoves[i] = make_int3(g, mv.y, mv.z);
-        const int cell = partition_of(I, inst, bits, o);
+        const int cell = head || far2 > 0.0 ? partition_of(I, inst, bits, o) : 0;
         if (I.qhist) {
             // the re-divided quad-tree counts points at their positions after the step
             atomicSub(I.qhist + qt_fine(I, o), 1);
@@ -354,7 +359,7 @@ __global__ void k_intake_link(Dev d, const int3 *moves, int m, Inst I, int bits,
                 atomicCAS(d.status, 0, DEV_FAR);
             }
         }
-        next[i] = atomicExch(head + cell, i);
+        if (head) next[i] = atomicExch(head + cell, i);
     }
 }
 
@@ -606,6 +611,7 @@ __global__ void __launch_bounds__(WPB * 32, MINB) k_kinetic(Dev dp, const int3 *
                                                             int4 *deferred, int *defer_count, int defer_cap,
                                                             int *viol, int viol_cap)
 {
+    if (I.pending && __ldcg(I.pending) == 0) return;  // the rounds did every move
     KD_BLOCK_DEV(dp);
     __shared__ WarpShared shs[WPB];
     int wib = threadIdx.x >> 5;
@@ -996,54 +1002,12 @@ __global__ void k_init(Dev d, const int *order, const int *third, int *tri_count
     *tri_count = s0 + 4;
 }
 
-// Insert the points at sorted positions (2j+1) * 2^level, each starting its walk at
-// the triangle of its Hilbert predecessor (2j) * 2^level, already inserted.
-__global__ void __launch_bounds__(WPB * 32) k_insert_level(Dev dp, const int *order, int level, int items,
-                                                           int *tri_count, int nloc, int slot_end)
-{
-    KD_BLOCK_DEV(dp);
-    __shared__ WarpShared shs[WPB];
-    int wib = threadIdx.x >> 5;
-    int gw = blockIdx.x * (blockDim.x >> 5) + wib;
-    int nw = gridDim.x * (blockDim.x >> 5);
-    Warp w = make_warp(&shs[wib], gw + 1, gw * 7 + level * 1315423911u, d);
-    // each warp takes a contiguous run of the level's points: runs are far apart along
-    // the Hilbert curve, so the insertions in flight at any moment rarely share a cavity
-    const int per = (items + nw - 1) / nw;
-    const int jend = min(items, (gw + 1) * per);
-    for (int j = gw * per; j < jend; ++j) {
-        if (read_status(d)) break;
-        long long i = ((long long)(2 * j + 1)) << level;
-        if (i >= nloc) continue;
-        int v = order[i];
-        if (__shfl_sync(FULL, __ldcg(d.pt_tri + v), 0) >= 0) continue;  // one of the first three
-        int parent = order[i - (1ll << level)];
-        int start = __shfl_sync(FULL, __ldcg(d.pt_tri + parent), 0);
-        if (start < 0) start = 0;
-        int s = 0;
-        if (w.lane == 0) s = atomicAdd(tri_count, 2);
-        s = __shfl_sync(FULL, s, 0);
-        if (s + 1 >= slot_end) {
-            set_status(d, DEV_INTERNAL);
-            break;
-        }
-        int2 q = d.xy[v];
-        int rc = insert_staged(w, d, v, q, start, s, s + 1, false);
-        if (rc == INS_GLOBAL) rc = insert_point(w, d, v, q, start, s, s + 1, false);
-        if (rc) {
-            if (rc > 0) set_status(d, rc);
-            break;
-        }
-    }
-    flush_counters(w, d);
-}
-
 // ------------------------------------------------------------------ batched build
 //
 // All instances of a batch built by one set of launches: per-instance bounding boxes,
 // Hilbert keys offset by instance (so one counting sort orders every instance's points
-// inside its own range of `order`), per-instance first triangles, and one launch per
-// insertion level whose items are every instance's points of that level, back to back.
+// inside its own range of `order`), per-instance first triangles, and rounds of insertions
+// over all instances (kdt_rounds.cuh), level by level.
 
 // bounding box of every instance (bbox[4 i .. 4 i + 3]) and the range check
 __global__ void k_range_batch(const int2 *xy, int n, const int *pofs, int ninst, int bits, int *status, int *bbox)
@@ -1119,58 +1083,6 @@ __global__ void k_init_batch(Dev d, const int *order, const int *third, const in
         d.pt_tri[c] = t0;
         tri_count[i] = s0 + 4;
     }
-}
-
-// One insertion level of every instance: items lvoff[i] .. lvoff[i+1]-1 are instance
-// i's points at its sorted positions (2j+1) * 2^level (as k_insert_level); each warp
-// takes a contiguous run of the items, so its insertions are far apart along their
-// instance's Hilbert curve.
-__global__ void __launch_bounds__(WPB * 32) k_insert_level_batch(Dev dp, const int *order, int level, int items,
-                                                                 const int *lvoff, const int *pofs, const int *tofs,
-                                                                 int ninst, int *tri_count)
-{
-    KD_BLOCK_DEV(dp);
-    __shared__ WarpShared shs[WPB];
-    int wib = threadIdx.x >> 5;
-    int gw = blockIdx.x * (blockDim.x >> 5) + wib;
-    int nw = gridDim.x * (blockDim.x >> 5);
-    Warp w = make_warp(&shs[wib], gw + 1, gw * 7 + level * 1315423911u, d);
-    const int per = (items + nw - 1) / nw;
-    const int gend = min(items, (gw + 1) * per);
-    int cur = -1, p0 = 0, nloc = 0;
-    for (int g = gw * per; g < gend; ++g) {
-        if (read_status(d)) break;
-        const int inst = csr_find(lvoff, ninst + 1, g);
-        if (inst != cur) {
-            cur = inst;
-            p0 = pofs[inst];
-            nloc = pofs[inst + 1] - p0;
-            set_instance(w, p0, nloc);
-        }
-        const int j = g - lvoff[inst];
-        long long i = ((long long)(2 * j + 1)) << level;
-        if (i >= nloc) continue;
-        int v = order[p0 + i];
-        if (__shfl_sync(FULL, __ldcg(d.pt_tri + v), 0) >= 0) continue;  // one of the first three
-        int parent = order[p0 + i - (1ll << level)];
-        int start = __shfl_sync(FULL, __ldcg(d.pt_tri + parent), 0);
-        if (start < 0) start = tofs[inst];
-        int s = 0;
-        if (w.lane == 0) s = atomicAdd(tri_count + inst, 2);
-        s = __shfl_sync(FULL, s, 0);
-        if (s + 1 >= tofs[inst + 1]) {
-            set_status(d, DEV_INTERNAL);
-            break;
-        }
-        int2 q = d.xy[v];
-        int rc = insert_staged(w, d, v, q, start, s, s + 1, false);
-        if (rc == INS_GLOBAL) rc = insert_point(w, d, v, q, start, s, s + 1, false);
-        if (rc) {
-            if (rc > 0) set_status(d, rc);
-            break;
-        }
-    }
-    flush_counters(w, d);
 }
 
 // ------------------------------------------------------------------ export
