@@ -86,7 +86,7 @@ struct kdt {
     int *scan_tmp = nullptr;
     int scan_tmp_cap = 0;
     // build / export temporaries (kept between calls)
-    Buf key, bord, hist, hoff, exp_cnt, exp_off, exp_fill, exp_out;
+    Buf key, bord, hist, hoff, exp_cnt, exp_off, exp_fill, exp_out, exp_rows;
     Buf btab, blev;  // batched build: per-instance tables, per-level item offsets
     // rounds (kdt_rounds.cuh): of a build, and of the steps (sized for mcap moves)
     Buf rb_cnt, rb_lost, rb_hdr, rb_rec, rb_queue, rb_left;
@@ -851,7 +851,7 @@ void free_state(kdt *h)
     h->ppart = nullptr;
     h->qleaves = 0;
     h->mcap = 0; h->dirty_cap = 0; h->scan_tmp_cap = 0; h->rm_rounds = 0;
-    Buf *bs[] = {&h->key, &h->bord, &h->hist, &h->hoff, &h->exp_cnt, &h->exp_off, &h->exp_fill, &h->exp_out,
+    Buf *bs[] = {&h->key, &h->bord, &h->hist, &h->hoff, &h->exp_cnt, &h->exp_off, &h->exp_fill, &h->exp_out, &h->exp_rows,
                  &h->btab, &h->blev, &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left,
                  &h->rm_cnt, &h->rm_lost, &h->rm_hdr, &h->rm_rec, &h->rm_slots, &h->rm_left,
                  &h->nb_deg, &h->nb_off, &h->nb_list, &h->dc_dist, &h->dc_cmin, &h->dc_scal};
@@ -1381,8 +1381,9 @@ int step_core(kdt *h, const kdt_move *moves, const int64_t *moff, int64_t m)
     return KDT_OK;
 }
 
-// canonical export of slots [s0, s0 + nslots) whose point ids are idbase .. idbase + np - 1
-int export_range(kdt *h, int s0, int nslots, int idbase, int np, int32_t *out, int64_t cap, int64_t *n_tri)
+// Canonical export of slots [s0, s0 + nslots) whose point ids are idbase .. idbase + np - 1,
+// by placing every row (any degrees).
+int export_placed(kdt *h, int s0, int nslots, int idbase, int np, int32_t *out, int64_t cap, int64_t *n_tri)
 {
     cudaStream_t st = h->stream;
     if (grow(h->exp_cnt, (size_t)np * 4) || grow(h->exp_off, (size_t)np * 4) || grow(h->exp_fill, (size_t)np * 4))
@@ -1412,6 +1413,48 @@ int export_range(kdt *h, int s0, int nslots, int idbase, int np, int32_t *out, i
     if (!dev_out && total > 0)
         CK(cudaMemcpyAsync(out, dst, (size_t)total * sizeof(int3), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    return KDT_OK;
+}
+
+// The same in buckets of first ids (k_exb_*): the default.  A bucket with more rows than its
+// block holds (first ids whose degrees are far above the mean) takes export_placed.
+int export_range(kdt *h, int s0, int nslots, int idbase, int np, int32_t *out, int64_t cap, int64_t *n_tri)
+{
+    cudaStream_t st = h->stream;
+    int s = 4;
+    while (s < EXB_SHIFT && (np >> s) > 2048) ++s;
+    const int nb = ((np - 1) >> s) + 1;
+    const bool dev_out = cap > 0 && on_device(h, out);
+    const int64_t room = std::min<int64_t>(cap, 2 * (int64_t)np);  // (2 np - 5 rows at most)
+    if (grow(h->exp_cnt, ((size_t)(EXB_PAD + 1) * nb + 1) * sizeof(int)) ||
+        (cap > 0 && grow(h->exp_rows, (size_t)std::max<int64_t>(room, 1) * sizeof(int3))) ||
+        (cap > 0 && !dev_out && grow(h->exp_out, (size_t)room * sizeof(int3))))
+        return KDT_ERR_CUDA;
+    int *cnt = (int *)h->exp_cnt.p, *off = cnt + (size_t)EXB_PAD * nb;
+    int *total = h->scal + S_TOTAL, *most = h->scal + S_MOST;
+    const TriHalf tv{h->tri + 2 * (size_t)s0};
+    CK(cudaMemsetAsync(cnt, 0, (size_t)EXB_PAD * nb * sizeof(int), st));
+    k_exb_count<<<thread_grid(h, nslots, 256), 256, 0, st>>>(tv, nslots, cnt, idbase, s);
+    k_exb_scan<<<1, 1024, 0, st>>>(cnt, nb, off, total, most);
+    h->stats.kernel_launches += 2;
+    int32_t *dst = dev_out ? out : (int32_t *)h->exp_out.p;
+    if (cap > 0) {
+        const size_t smem = ((2 + 3 * (size_t)EXB_ROWS) << s) * sizeof(int);
+        k_exb_append<<<thread_grid(h, nslots, 256), 256, 0, st>>>(tv, nslots, cnt, (int3 *)h->exp_rows.p, idbase, s, total,
+                                                                 most, cap);
+        k_exb_sort<<<nb, EXB_THREADS, smem, st>>>((const int3 *)h->exp_rows.p, off, s, dst, total, most, cap);
+        h->stats.kernel_launches += 2;
+    }
+    CK(cudaGetLastError());
+    if (sync_scalars(h)) return KDT_ERR_CUDA;
+    *n_tri = h->hscal[S_TOTAL];
+    if (*n_tri > cap) return KDT_ERR_CAPACITY;
+    if (*n_tri == 0) return KDT_OK;
+    if (h->hscal[S_MOST] > EXB_ROWS << s) return export_placed(h, s0, nslots, idbase, np, out, cap, n_tri);
+    if (!dev_out) {
+        CK(cudaMemcpyAsync(out, dst, (size_t)*n_tri * sizeof(int3), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+    }
     return KDT_OK;
 }
 
@@ -1613,7 +1656,9 @@ int kdt_create(kdt **out, const kdt_config *cfg, int device, void *cuda_stream)
     cudaMemset(h->counters, 0, C_SLOTS * sizeof(unsigned long long));
     if (cudaFuncSetAttribute(k_mlp_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TCS_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_mlp_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TCS_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(k_mlp_grad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TG_BYTES) != cudaSuccess) {
+        cudaFuncSetAttribute(k_mlp_grad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TG_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_exb_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(((2 + 3 * EXB_ROWS) << EXB_SHIFT) * sizeof(int))) != cudaSuccess) {
         kdt_destroy(h);
         return KDT_ERR_CUDA;
     }

@@ -118,3 +118,32 @@ def test_more_moves_than_a_round():
     assert np.array_equal(t.export_points(), xy)
     assert t.verify() == 0
     assert t.stats()["rebuilds"] == 1
+
+
+@pytest.mark.parametrize("n,hub", [(3, 0), (15, 0), (16, 0), (17, 0), (4097, 0), (33000, 0), (600, 500), (40000, 9000)])
+def test_export_buckets(n, hub):
+    """The export in buckets of first ids: one bucket, its last id, several ids a bucket; and a
+    bucket with more rows than its block holds (a fan of `hub` triangles around id 0), which
+    is placed instead.  Into host and device memory, and with too little room."""
+    import torch
+    from paper_2308_06484_gb300 import kdt
+    if hub:
+        a = np.pi * np.arange(hub) / (hub - 1)
+        rim = np.stack([(1 << 27) + 1e8 * np.cos(a), (1 << 26) + 1e8 * np.sin(a)], 1)
+        rest = W.uniform_points(n - hub - 1, 20, 3)
+        xy = np.concatenate([[[1 << 27, 1 << 26]], np.rint(rim), rest]).astype(np.int32)
+        xy = np.concatenate([xy[:1], np.unique(xy[1:], axis=0)])
+    else:
+        xy = W.uniform_points(n, 24, n)
+    t = _tri(domain_bits=28)
+    t.build(np.ascontiguousarray(xy))
+    got = t.export_triangles()
+    assert_same(got, xy, "export n=%d" % n)
+    out = torch.full((2 * len(xy), 3), -1, dtype=torch.int32, device="cuda")
+    assert np.array_equal(t.export_triangles(out).cpu().numpy(), got)
+    assert int((out[got.shape[0]:] != -1).sum()) == 0
+    out.fill_(-1)
+    if got.shape[0] > 1:
+        with pytest.raises(kdt.KDTError) as e:
+            t.export_triangles(out[:got.shape[0] - 1])
+        assert e.value.name == "KDT_ERR_CAPACITY" and int((out != -1).sum()) == 0
