@@ -1075,7 +1075,7 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
                                                              net ? h->pguess : nullptr, ordered ? h->pcost : nullptr,
                                                              tensor ? h->pfeat : nullptr, tensor ? h->ppart : nullptr);
         if (tensor)
-            k_mlp_tc<1><<<tc_grid(h, cap), TC_M, TCS_BYTES, st>>>(h->mlp_w, h->pfeat, mi, from_ctl ? h->ctl : nullptr,
+            k_mlp_tc<1><<<tc_grid(h, cap), TC_THREADS, TCS_BYTES, st>>>(h->mlp_w, h->pfeat, mi, from_ctl ? h->ctl : nullptr,
                                                                   nullptr, h->ppart, h->gmoves, h->pguess,
                                                                   ordered ? h->pcost : nullptr,
                                                                   h->counters + C_TC_FAIL);
@@ -2084,7 +2084,7 @@ int kdt_mlp_forward_tc(kdt *h, const uint16_t *params_bf16, const float *x, int6
     CK(cudaSetDevice(h->device));
     if (!on_device(h, params_bf16) || !on_device(h, x) || !on_device(h, out)) return KDT_ERR_ARG;
     if (((uintptr_t)params_bf16 & 3) != 0) return KDT_ERR_ARG;  // weight rows read as BF16 pairs
-    k_mlp_tc<0><<<tc_grid(h, rows), TC_M, TCS_BYTES, h->stream>>>((const unsigned short *)params_bf16, x, rows,
+    k_mlp_tc<0><<<tc_grid(h, rows), TC_THREADS, TCS_BYTES, h->stream>>>((const unsigned short *)params_bf16, x, rows,
                                                                   nullptr, out, nullptr, nullptr, nullptr, nullptr,
                                                                   h->counters + C_TC_FAIL);
     h->stats.kernel_launches++;
@@ -2122,7 +2122,7 @@ int kdt_mlp_loss_grad(kdt *h, const uint16_t *params_bf16, const float *x, const
     float *part_loss = h->mlp_part + (size_t)h->mlp_part_blocks * MLP_PARAMS;
     k_mlp_grad<<<blocks, GTHREADS, smem, h->stream>>>((const unsigned short *)params_bf16, x, (const int *)labels,
                                                      (const long long *)index, rows, lam, h->mlp_part, part_loss);
-    k_mlp_reduce<<<(MLP_PARAMS + 255) / 256, 256, 0, h->stream>>>(h->mlp_part, part_loss, blocks, rows, grad, loss);
+    k_mlp_reduce<<<REDUCE_BLOCKS, 32 * REDUCE_WARPS, 0, h->stream>>>(h->mlp_part, part_loss, blocks, rows, grad, loss);
     h->stats.kernel_launches += 2;
     CK(cudaGetLastError());
     return KDT_OK;
@@ -2140,10 +2140,10 @@ int kdt_mlp_loss_grad_tc(kdt *h, const uint16_t *params_bf16, const float *x, co
     const int blocks = (int)std::min<long long>((rows + TC_M - 1) / TC_M, sm_count(h->device));
     if (int rc = ensure_mlp_part(h, blocks)) return rc;
     float *part_loss = h->mlp_part + (size_t)h->mlp_part_blocks * MLP_PARAMS;
-    k_mlp_grad_tc<<<blocks, TC_M, TG_BYTES, h->stream>>>((const unsigned short *)params_bf16, x, (const int *)labels,
+    k_mlp_grad_tc<<<blocks, TG_THREADS, TG_BYTES, h->stream>>>((const unsigned short *)params_bf16, x, (const int *)labels,
                                                         (const long long *)index, rows, lam, h->mlp_part, part_loss,
                                                         h->counters + C_TC_FAIL);
-    k_mlp_reduce<<<(MLP_PARAMS + 255) / 256, 256, 0, h->stream>>>(h->mlp_part, part_loss, blocks, rows, grad, loss);
+    k_mlp_reduce<<<REDUCE_BLOCKS, 32 * REDUCE_WARPS, 0, h->stream>>>(h->mlp_part, part_loss, blocks, rows, grad, loss);
     h->stats.kernel_launches += 2;
     CK(cudaGetLastError());
     return KDT_OK;

@@ -275,20 +275,43 @@ __global__ void __launch_bounds__(GTHREADS) k_mlp_grad(const unsigned short *wb,
     if (tid == 0) partial_loss[blockIdx.x] = lsum;
 }
 
-// grad[i] = sum over blocks of partial[b][i] in block order; loss likewise (divided by rows).
-__global__ void k_mlp_reduce(const float *partial, const float *partial_loss, int nblocks, long long rows, float *grad,
-                             float *loss)
+constexpr int REDUCE_WARPS = 8;  // of k_mlp_reduce: slices of the partials
+constexpr int REDUCE_BLOCKS = (MLP_PARAMS + 31) / 32;
+
+// grad[i] = the sum of the blocks' partials, 32 parameters per block: warp s adds the s-th
+// slice of the partials in block order (neighbouring parameters, so 128-byte reads; one
+// thread adding all of 152 partials waits for each in turn), then the slices in order.
+// loss likewise (divided by rows).  Fixed order: the result repeats exactly.
+__global__ void __launch_bounds__(32 * REDUCE_WARPS) k_mlp_reduce(const float *partial, const float *partial_loss,
+                                                                  int nblocks, long long rows, float *grad, float *loss)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ float sum[REDUCE_WARPS][33];
+    const int lane = threadIdx.x & 31, s = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    const int per = (nblocks + REDUCE_WARPS - 1) / REDUCE_WARPS, lo = s * per, hi = min(nblocks, lo + per);
+    float g = 0.f;
     if (i < MLP_PARAMS) {
-        float g = 0.f;
-        for (int b = 0; b < nblocks; ++b) g += partial[(long long)b * MLP_PARAMS + i];
-        grad[i] = g;
+#pragma unroll 8
+        for (int b = lo; b < hi; ++b) g += __ldg(partial + (long long)b * MLP_PARAMS + i);
+    }
+    sum[s][lane] = g;
+    if (lane == 0) {
+        float l = 0.f;
+        if (blockIdx.x == 0 && loss)
+            for (int b = lo; b < hi; ++b) l += __ldg(partial_loss + b);
+        sum[s][32] = l;
+    }
+    __syncthreads();
+    if (s != 0) return;
+    if (i < MLP_PARAMS) {
+        float t = sum[0][lane];
+#pragma unroll
+        for (int k = 1; k < REDUCE_WARPS; ++k) t += sum[k][lane];
+        grad[i] = t;
     }
     if (i == 0 && loss) {
-        float l = 0.f;
-        for (int b = 0; b < nblocks; ++b) l += partial_loss[b];
-        *loss = l / (float)rows;
+        float t = sum[0][32];
+        for (int k = 1; k < REDUCE_WARPS; ++k) t += sum[k][32];
+        *loss = t / (float)rows;
     }
 }
 
