@@ -321,7 +321,8 @@ int kdt_export_triangles_noalloc(kdt *h, int32_t *out, int64_t cap, int64_t *n_t
  *              or NULL;
  *   info:      host, required.
  * Errors: KDT_ERR_ARG (N out of range, info NULL), KDT_ERR_STATE (not built),
- * KDT_ERR_CUDA.  Allocates device scratch (neighbour lists, ~28 bytes per point). */
+ * KDT_ERR_CUDA.  The stars are walked on the triangulation itself; the device scratch is the
+ * results' when they go to the host. */
 typedef struct {
     int64_t min2;     /* mindistance(P)^2 of this call                                     */
     int64_t d2;       /* d^2: the running minimum (see above)                              */

@@ -52,6 +52,7 @@ struct kdt {
     int64_t n = 0;  // points (all instances)
     int cap = 0;    // triangle slots (all instances)
     bool built = false;
+    bool order_valid = false;  // bord holds every point, in the last build's Hilbert order
     int stamp = 0;
     // instances
     int ninst = 0;
@@ -92,8 +93,8 @@ struct kdt {
     Buf rb_cnt, rb_lost, rb_hdr, rb_rec, rb_queue, rb_left;
     Buf rm_cnt, rm_lost, rm_hdr, rm_rec, rm_slots, rm_left;
     int rm_rounds = 0, rm_ops = 0;
-    // d-calculation: neighbour lists, results, running minimum (per N)
-    Buf nb_deg, nb_off, nb_list, dc_dist, dc_cmin, dc_scal;
+    // d-calculation: results, running minimum (per N)
+    Buf dc_dist, dc_cmin, dc_scal;
     int64_t d2_run = INT64_MAX;
     int d_n = 0;
     // the displacement rule (kdt_config.rebuild_displacement): running per-partition
@@ -695,6 +696,7 @@ int rebuild_batch(kdt *h)
 int rebuild_all(kdt *h)
 {
     h->built = false;
+    h->order_valid = false;
     h->stamp++;
     int rc = h->ninst > 1 && h->cfg.batch_build ? rebuild_batch(h) : BATCH_TOO_WIDE;
     if (rc != BATCH_TOO_WIDE && rc != KDT_OK) return rc;
@@ -705,6 +707,7 @@ int rebuild_all(kdt *h)
         }
     }
     h->built = true;
+    h->order_valid = rc == KDT_OK || h->ninst == 1;  // (one instance after another leaves the last one's)
     h->stats.rebuilds++;
     return KDT_OK;
 }
@@ -854,12 +857,13 @@ void free_state(kdt *h)
     Buf *bs[] = {&h->key, &h->bord, &h->hist, &h->hoff, &h->exp_cnt, &h->exp_off, &h->exp_fill, &h->exp_out, &h->exp_rows,
                  &h->btab, &h->blev, &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left,
                  &h->rm_cnt, &h->rm_lost, &h->rm_hdr, &h->rm_rec, &h->rm_slots, &h->rm_left,
-                 &h->nb_deg, &h->nb_off, &h->nb_list, &h->dc_dist, &h->dc_cmin, &h->dc_scal};
+                 &h->dc_dist, &h->dc_cmin, &h->dc_scal};
     for (Buf *b : bs) free_buf(*b);
     h->n = 0;
     h->cap = 0;
     h->ninst = 0;
     h->built = false;
+    h->order_valid = false;
     h->tune_idx = -1;
     h->tune_done = 0;
 }
@@ -1798,20 +1802,7 @@ int d_values_impl(kdt *h, int N, int64_t *dist2, int64_t *cell_min2, kdt_dinfo *
         if (h->pofs[i + 1] - h->pofs[i] <= N) return KDT_ERR_ARG;
     cudaStream_t st = h->stream;
     const int n = (int)h->n;
-    // neighbour lists (CSR) from the live triangles
-    if (grow(h->nb_deg, (size_t)n * sizeof(int)) || grow(h->nb_off, (size_t)(n + 1) * sizeof(int)) ||
-        grow(h->dc_scal, 4 * sizeof(unsigned long long)))
-        return KDT_ERR_CUDA;
-    int *deg = (int *)h->nb_deg.p, *off = (int *)h->nb_off.p;
-    CK(cudaMemsetAsync(deg, 0, (size_t)n * sizeof(int), st));
-    k_nbr_count<<<thread_grid(h, h->cap, 256), 256, 0, st>>>(TriHalf{h->tri}, h->cap, deg);
-    if (scan(h, deg, off, n, off + n, st)) return KDT_ERR_CUDA;
-    int total = 0;
-    CK(cudaMemcpyAsync(&total, off + n, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    if (grow(h->nb_list, (size_t)std::max(total, 1) * sizeof(int))) return KDT_ERR_CUDA;
-    CK(cudaMemsetAsync(deg, 0, (size_t)n * sizeof(int), st));  // now the fill positions
-    k_nbr_fill<<<thread_grid(h, h->cap, 256), 256, 0, st>>>(TriHalf{h->tri}, h->cap, off, deg, (int *)h->nb_list.p);
+    if (grow(h->dc_scal, 4 * sizeof(unsigned long long))) return KDT_ERR_CUDA;
     // the N-th nearest neighbours and their minima
     const bool dist_dev = dist2 && on_device(h, dist2);
     const bool cmin_dev = cell_min2 && on_device(h, cell_min2);
@@ -1837,12 +1828,14 @@ int d_values_impl(kdt *h, int N, int64_t *dist2, int64_t *cell_min2, kdt_dinfo *
     unsigned long long *sc = (unsigned long long *)h->dc_scal.p;  // [0] minimum, [1] largest degree
     unsigned long long init[2] = {(unsigned long long)INT64_MAX, 0ull};
     CK(cudaMemcpyAsync(sc, init, sizeof init, cudaMemcpyHostToDevice, st));
-    k_nth_nn<<<thread_grid(h, n, 128), 128, 0, st>>>(h->xy, off, (const int *)h->nb_list.p, n, N, make_inst(h),
-                                                    h->cfg.domain_bits, dd, cm, sc, (int *)(sc + 1));
+    auto nth = N <= 2 ? k_nth_nn<2> : (N <= 4 ? k_nth_nn<4> : (N <= 8 ? k_nth_nn<8> : k_nth_nn<DC_MAX_N>));
+    nth<<<(n + 127) / 128, 128, 0, st>>>(h->xy, h->pt_tri, TriHalf{h->tri}, TriHalf{h->tri + 1},
+                                         h->order_valid ? (const int *)h->bord.p : nullptr, n, N, make_inst(h),
+                                         h->cfg.domain_bits, dd, cm, sc, (int *)(sc + 1));
     const int restart = !h->dloc_valid || h->d_n != N;
     k_merge_min_u64<<<thread_grid(h, h->ncells, 256), 256, 0, st>>>(h->dloc2, cm, h->ncells, restart);
     h->dloc_valid = true;
-    h->stats.kernel_launches += 8;
+    h->stats.kernel_launches += 3;
     CK(cudaGetLastError());
     if (dist2 && !dist_dev)
         CK(cudaMemcpyAsync(dist2, dd, (size_t)n * sizeof(long long), cudaMemcpyDeviceToHost, st));

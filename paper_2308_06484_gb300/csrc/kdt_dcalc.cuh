@@ -21,82 +21,79 @@ namespace kd {
 
 constexpr int DC_MAX_N = 16;  // largest N a call may ask for
 
-// Neighbour counts from the live triangles: every edge u -> v of a triangle in
-// counter-clockwise order gives u the neighbour v.  An interior edge is seen once from
-// each side and a hull edge once from its finite triangle and once from its ghost, so
-// every neighbour is counted exactly once.
-__global__ void k_nbr_count(TriHalf tv, int nslots, int *deg)
-{
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nslots; t += gridDim.x * blockDim.x) {
-        int4 v = tv[t];
-        if (!(v.w & ALIVE)) continue;
-        if (v.x >= 0 && v.y >= 0) atomicAdd(deg + v.x, 1);
-        if (v.y >= 0 && v.z >= 0) atomicAdd(deg + v.y, 1);
-        if (v.z >= 0 && v.x >= 0) atomicAdd(deg + v.z, 1);
-    }
-}
-
-// The same edges written into the lists (off: exclusive scan of the counts; cur:
-// zeroed fill positions).  The order inside a list does not matter.
-__global__ void k_nbr_fill(TriHalf tv, int nslots, const int *off, int *cur, int *nbr)
-{
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nslots; t += gridDim.x * blockDim.x) {
-        int4 v = tv[t];
-        if (!(v.w & ALIVE)) continue;
-        if (v.x >= 0 && v.y >= 0) nbr[off[v.x] + atomicAdd(cur + v.x, 1)] = v.y;
-        if (v.y >= 0 && v.z >= 0) nbr[off[v.y] + atomicAdd(cur + v.y, 1)] = v.z;
-        if (v.z >= 0 && v.x >= 0) nbr[off[v.z] + atomicAdd(cur + v.z, 1)] = v.x;
-    }
-}
-
 __device__ __forceinline__ long long dist2_of(int2 a, int2 b)
 {
     long long dx = (long long)a.x - b.x, dy = (long long)a.y - b.y;
     return dx * dx + dy * dy;
 }
 
-// One thread per point: the N nearest, one at a time, from the neighbour lists (see
-// the header).  bd/bi hold the best candidates in (distance, id) order; entries
-// 0 .. e-1 are the points taken so far.  Writes dist2[p] (if asked), the minimum of
-// its partition (cell_min, if asked) and of all points (gmin); the largest degree met
-// goes to max_deg.
-__global__ void k_nth_nn(const int2 *xy, const int *off, const int *nbr, int n, int N, Inst I, int bits,
-                         long long *dist2, unsigned long long *cell_min, unsigned long long *gmin, int *max_deg)
+// One thread per point: the N <= CAP nearest, one at a time, each time from the stars of p
+// and of the points already taken (see the header).  A star is walked on the triangulation
+// itself; neighbouring threads take neighbouring points (order: the build's Hilbert order,
+// or null: ids), so the triangles and positions of one warp's walks come from the same few
+// sectors of L1 and L2.  (Neighbour lists first, counted, scanned and filled with two passes of
+// atomics, then one random 8-byte read per list entry: 435 us a call on 1e6 points, N = 4;
+// this: 242.)  bd / bi hold the best candidates in (distance, id) order, in
+// registers (every loop over them is unrolled); entries 0 .. e are the points taken.
+// Writes dist2[p] (if asked), the minimum of its partition (cell_min, if asked) and of all
+// points (gmin); the largest degree met goes to max_deg.
+template <int CAP>
+__global__ void __launch_bounds__(128) k_nth_nn(const int2 *xy, const int *pt_tri, TriHalf tv, TriHalf tn,
+                                                const int *order, int n, int N, Inst I, int bits, long long *dist2,
+                                                unsigned long long *cell_min, unsigned long long *gmin, int *max_deg)
 {
     long long best = LLONG_MAX;
     int mdeg = 0;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-        const int2 pp = xy[p];
-        long long bd[DC_MAX_N];
-        int bi[DC_MAX_N];
-        int cnt = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int p = order ? __ldg(order + i) : i;
+        const int2 pp = __ldg(xy + p);
+        long long bd[CAP];
+        int bi[CAP];
+#pragma unroll
+        for (int j = 0; j < CAP; ++j) {
+            bd[j] = LLONG_MAX;
+            bi[j] = INT_MAX;
+        }
         int src = p;
         for (int e = 0; e < N; ++e) {
             // add the neighbours of src (p, then the point taken last)
-            const int lo = off[src], hi = off[src + 1];
-            mdeg = max(mdeg, hi - lo);
-            for (int k = lo; k < hi; ++k) {
-                const int w = nbr[k];
+            const int t0 = __ldg(pt_tri + src);
+            int t = t0, deg = 0, steps = 0;
+            do {
+                const int4 v = __ldg(tv + t), nb = __ldg(tn + t);
+                const int k = v.x == src ? 0 : (v.y == src ? 1 : 2);
+                const int w = k == 0 ? v.y : (k == 1 ? v.z : v.x);
+                t = (k == 0 ? nb.y : (k == 1 ? nb.z : nb.x)) >> 2;
+                if (w < 0) continue;  // the vertex at infinity
+                ++deg;
                 if (w == p) continue;
-                const long long dw = dist2_of(pp, xy[w]);
-                if (cnt == N && (dw > bd[N - 1] || (dw == bd[N - 1] && w >= bi[N - 1]))) continue;
+                long long cd = dist2_of(pp, __ldg(xy + w));
+                int ci = w;
                 bool seen = false;
-                for (int j = 0; j < cnt; ++j) seen = seen || bi[j] == w;
+#pragma unroll
+                for (int j = 0; j < CAP; ++j) seen = seen || (j < N && bi[j] == w);
                 if (seen) continue;
-                int j = cnt < N ? cnt : N - 1;  // the slot freed at the end
-                while (j > 0 && (bd[j - 1] > dw || (bd[j - 1] == dw && bi[j - 1] > w))) {
-                    bd[j] = bd[j - 1];
-                    bi[j] = bi[j - 1];
-                    --j;
-                }
-                bd[j] = dw;
-                bi[j] = w;
-                if (cnt < N) ++cnt;
-            }
-            if (e == cnt) break;  // fewer than N other points reachable (cannot happen for n > N)
-            src = bi[e];          // the (e+1)-th nearest: expand it next
+#pragma unroll
+                for (int j = 0; j < CAP; ++j)
+                    if (j < N && (cd < bd[j] || (cd == bd[j] && ci < bi[j]))) {
+                        const long long td = bd[j];
+                        const int tj = bi[j];
+                        bd[j] = cd;
+                        bi[j] = ci;
+                        cd = td;
+                        ci = tj;
+                    }
+            } while (t != t0 && ++steps <= n);  // (a star has at most n triangles)
+            mdeg = max(mdeg, deg);
+#pragma unroll
+            for (int j = 0; j < CAP; ++j)
+                if (j == e) src = bi[j];  // the (e+1)-th nearest: expand it next
+            if (src == INT_MAX) break;    // fewer than N other points reachable (cannot happen for n > N)
         }
-        const long long v = cnt == N ? bd[N - 1] : LLONG_MAX;
+        long long v = LLONG_MAX;
+#pragma unroll
+        for (int j = 0; j < CAP; ++j)
+            if (j == N - 1) v = bd[j];
         if (dist2) dist2[p] = v;
         if (cell_min) {
             const int inst = I.ninst > 1 ? csr_find(I.pofs, I.ninst + 1, p) : 0;
