@@ -424,17 +424,17 @@ Rounds make_rounds(const Buf &cnt, int rounds, const Buf &lost, const Buf &hdr, 
 
 // A round's kernels for at most `most` operations; wide: 32 lanes plan an operation (twice
 // the limits of 16 lanes, half the rate); last: what the plan cannot take is left out.
-template <bool MOVE>
+template <int MODE>
 void launch_round(kdt *h, cudaStream_t st, const Dev &d, const Rounds &R, int b, long long most, const RoundMoves &M,
                   const RoundBuild &B, bool wide, bool last)
 {
     const int sms = sm_count(h->device);
     // (a warp for every operation, while the GPU has room for that many)
     const long long pb = std::min<long long>((most * 32 + ROUND_THREADS - 1) / ROUND_THREADS, 32ll * sms);
-    auto plan = wide ? k_round_plan<MOVE, 32> : k_round_plan<MOVE, 16>;
+    auto plan = wide ? k_round_plan<MODE, 32> : k_round_plan<MODE, 16>;
     plan<<<(int)std::max(1ll, pb), ROUND_THREADS, 0, st>>>(d, R, b, M, B, last ? 1 : 0);
     const long long cb = std::min<long long>((most * ROUND_LANES + 255) / 256, 8ll * sms);
-    k_round_commit<MOVE><<<(int)std::max(1ll, cb), 256, 0, st>>>(d, R, b, M, B);
+    k_round_commit<MODE != REGION_INSERT><<<(int)std::max(1ll, cb), 256, 0, st>>>(d, R, b, M, B);
 }
 
 // A round of a build takes up to one BUILD_DIV-th as many new points as are in, or as many as
@@ -491,7 +491,7 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
         for (int i = 0; i < batch; ++i, ++b) {
             const long long most = std::min<long long>(
                 ops, std::max<long long>(64, std::max<long long>(in / BUILD_DIV, std::min<long long>(in, BUILD_FEW))));
-            launch_round<false>(h, st, d, R, b, most, M, B, wide, false);
+            launch_round<REGION_INSERT>(h, st, d, R, b, most, M, B, wide, false);
             in = std::min(in + most, np);
         }
         h->stats.kernel_launches += 2 * batch;
@@ -739,11 +739,13 @@ int ensure_moves(kdt *h, int64_t m)
 // it costs 20.
 constexpr int STEP_EXTRA_ROUNDS = 2, STEP_EXTRA_ROUNDS_MANY = 4, STEP_MANY = 32768;
 
-// Do the step's moves go through rounds?  The paper's method (delete and insert) without
-// training rows, proposal or planner; else the kinetic kernel does every move.
+// Do the step's moves go through rounds?  The paper's method (delete and insert), without
+// training rows and with no proposal or one the planner evaluates; else the kinetic kernel
+// does every move.
 bool step_in_rounds(const kdt *h)
 {
-    return h->cfg.variant == 0 && h->cfg.plan == 0 && !h->prop_on && !h->trace_x && h->cfg.kinetic_warps == 0;
+    return h->cfg.variant == 0 && (!h->prop_on || (h->cfg.plan & PLAN_NETWORK)) && !h->trace_x &&
+           h->cfg.kinetic_warps == 0;
 }
 
 int ensure_rounds(kdt *h)
@@ -1100,8 +1102,9 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
         R.left = (int *)h->rm_left.p;
         const RoundMoves M{h->gmoves};
         const RoundBuild B{nullptr, nullptr, nullptr, nullptr, nullptr, 0, mi, 0};
+        auto launch_moves = d.pguess ? launch_round<REGION_GUESS> : launch_round<REGION_MOVE>;
         for (int b = 0; b < h->rm_rounds; ++b)
-            launch_round<true>(h, st, d, R, b, std::min(cap, h->rm_ops), M, B, b + 1 == h->rm_rounds,
+            launch_moves(h, st, d, R, b, std::min(cap, h->rm_ops), M, B, b + 1 == h->rm_rounds,
                                b + 1 == h->rm_rounds);
         k_round_clear<<<thread_grid(h, (long long)cap * (RT / 4), 256), 256, 0, st>>>(
             d, R, h->rm_rounds, mi, I, h->cfg.domain_bits, h->gmoves, h->old_xy, h->head, h->next);

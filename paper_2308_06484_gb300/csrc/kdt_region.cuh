@@ -39,6 +39,7 @@ namespace kd {
 constexpr int RT = 32;     // most triangles an operation writes
 constexpr int RWALK = 1 << 12;  // steps of a walk before the operation is left to the other path
 
+enum RegionMode : int { REGION_INSERT = 0, REGION_MOVE = 1, REGION_GUESS = 2 };
 enum RegionResult : int { RG_OK = 0, RG_BAIL = 1, RG_VERTEX = 2 };
 
 // What the RL lanes of an operation share (RL: also the largest degree, cavity and border).
@@ -61,6 +62,7 @@ struct RegionOut {
     int t0;           // a triangle of the store near q (the next attempt's start), or -1
     unsigned ex, ti;  // exact predicate calls, ties (this lane's)
     int steps;        // triangles walked through
+    int prop;         // the learned proposal: 0 none, 1 a guess, 3 a guess whose triangle holds q
 };
 
 __device__ __forceinline__ int rcomp(const int4 &v, int i) { return i == 0 ? v.x : (i == 1 ? v.y : v.z); }
@@ -78,16 +80,18 @@ __device__ __forceinline__ int bit_prev(unsigned m, int i)
     return 31 - __clz((int)(a ? a : m));
 }
 
-// MOVE: delete p (its position is still the old one in d.xy) and insert it at q.
-// Otherwise insert p at q, walking from slot `start`, with the dead slots spare0, spare1.
+// MODE REGION_MOVE: delete p (its position is still the old one in d.xy) and insert it at q;
+// REGION_GUESS: the same with the learned proposal's guess as the locate's first candidate.
+// REGION_INSERT: insert p at q, walking from slot `start`, with the dead slots spare0, spare1.
 // All RL lanes of the group (lane l, member mask gm, first lane g0 of the warp) call with
 // the same arguments.  out[2 r], out[2 r + 1] receive triangle r < nt: (v0, v1, v2, alive
 // flag 1) and (n0, n1, n2, slot); a neighbour outside the region is stored as the
 // complement of its reference (its back reference has to follow).  sh.pool holds the slots.
-template <bool MOVE, int RL, class D>
+template <int MODE, int RL, class D>
 __device__ __forceinline__ int region_plan(const D &d, RegionShared<RL> &sh, int l, unsigned gm, int g0, int p, int2 q,
                                            int start, int spare0, int spare1, int4 *out, RegionOut &o)
 {
+    constexpr bool MOVE = MODE != REGION_INSERT;
     const int2 zero = make_int2(0, 0);
     auto sh1 = [&](int v, int src) { return __shfl_sync(gm, v, src, RL); };
     auto sh2 = [&](int2 v, int src) { return make_int2(__shfl_sync(gm, v.x, src, RL), __shfl_sync(gm, v.y, src, RL)); };
@@ -103,6 +107,7 @@ __device__ __forceinline__ int region_plan(const D &d, RegionShared<RL> &sh, int
     o.ex = 0;
     o.ti = 0;
     o.steps = 0;
+    o.prop = 0;
     int k = 0;
     // this lane's link vertex, its successor, its star triangle, the ring behind its link edge
     int id = -1, idn = -1, S = -1, O = 0, A = -1;
@@ -252,7 +257,30 @@ __device__ __forceinline__ int region_plan(const D &d, RegionShared<RL> &sh, int
         xa = sh2(x, ta);
         xb = sh2(x, tb3);
         xc = sh2(x, tc);
-        // ---- 2. locate q in the hole
+        // the learned proposal's guess (made by the step planner for this move): the rank of
+        // the hole triangle it names, as hole_rank and move_wedge define it.  (1e6 points,
+        // 4096 moves, planner on the tensor cores: 190 us a step with one warp a move, 121 so.)
+        int rank = -1, guess = -2;
+        if constexpr (MODE == REGION_GUESS) if (!gh) {
+            const int2 po = __ldcg(d.xy + p);
+            const long long dx = (long long)q.x - po.x, dy = (long long)q.y - po.y;
+            const long long ax = (long long)x.x - po.x, ay = (long long)x.y - po.y;
+            const long long bx = (long long)xn.x - po.x, by = (long long)xn.y - po.y;
+            const unsigned wm = votes(inl && ax * dy - ay * dx >= 0 && dx * by - dy * bx > 0);
+            if (__popc(wm) == 1) {
+                const int j0 = __ffs((int)wm) - 1;
+                const int ra = ta - j0 < 0 ? ta - j0 + k : ta - j0, rb = tb3 - j0 < 0 ? tb3 - j0 + k : tb3 - j0,
+                          rc = tc - j0 < 0 ? tc - j0 + k : tc - j0;
+                const int lo = min(ra, min(rb, rc)), hi = max(ra, max(rb, rc)), mid = ra + rb + rc - lo - hi;
+                const int key = lo << 12 | mid << 6 | hi;
+                rank = 0;
+                for (unsigned b = HM; b; b &= b - 1u) rank += sh1(key, __ffs((int)b) - 1) < key;
+                if (!has) rank = -1;
+                guess = (int)__ldcg(d.pguess + p);
+                o.prop = 1;
+            }
+        }
+        // ---- 2. locate q in the hole (first the triangle the proposal names)
         {
             bool in = false, out_ = false;
             int zeros = 0, vt = -1;
@@ -266,7 +294,12 @@ __device__ __forceinline__ int region_plan(const D &d, RegionShared<RL> &sh, int
                     out_ = orient2d(ia < 0 ? xb : (ib < 0 ? xc : xa), ia < 0 ? xc : (ib < 0 ? xa : xb), q) > 0;
                 }
             }
-            const unsigned inm = votes(in), om = votes(out_);
+            unsigned inm = votes(in);
+            const unsigned om = votes(out_), pm = o.prop ? votes(in && zeros < 2 && rank == guess) : 0u;
+            if (pm) {
+                inm = pm;
+                o.prop = 3;
+            }
             if (inm) {
                 const int src = __ffs((int)inm) - 1;
                 zeros = sh1(zeros, src);

@@ -63,7 +63,7 @@ struct Rounds {
     int *lostcnt;   // [rounds + 1]
     int *lost[2];   // item ids
     int4 *hdr;      // per operation of the round: item, triangles (0: plan again, -1: left to the
-                    // other path), priority, k | ncav << 8 | edge << 24 | ghost << 25
+                    // other path), priority, k | ncav << 8 | edge << 24 | ghost << 25 | prop << 26
     int4 *rec;      // per operation of the round: RT triangles (region_plan's out)
     int *slots;     // moves only, per operation since the step's start: RT slots (-1: none)
     int *left;      // items for the warp-wide path
@@ -145,10 +145,11 @@ __device__ __forceinline__ int near_start(const Dev &d, const int *order, int n,
 // itself, so no warp is as long as the union of two operations' paths.  An operation
 // outside RL's limits is planned again, by the 32-lane form when LAST is set or later, and
 // with LAST goes to the list of the warp-wide path.
-template <bool MOVE, int RL>
+template <int MODE, int RL>
 __global__ void __launch_bounds__(ROUND_THREADS, ROUND_BLOCKS) k_round_plan(Dev d, Rounds R, int b, RoundMoves M, RoundBuild B,
                                                               int last)
 {
+    constexpr bool MOVE = MODE != REGION_INSERT;
     if (__ldcg(d.status)) return;
     __shared__ RegionShared<RL> shared[ROUND_THREADS / RL];
     int total = B.total;
@@ -178,10 +179,10 @@ __global__ void __launch_bounds__(ROUND_THREADS, ROUND_BLOCKS) k_round_plan(Dev 
         RegionOut o;
         int4 *rec = R.rec + (size_t)x * (2 * RT);
         int rc, p;
-        if (MOVE) {
+        if constexpr (MOVE) {
             const int3 mv = M.gmoves[item];
             p = mv.x;
-            rc = region_plan<true, RL>(d, sh, l, gm, g0, p, make_int2(mv.y, mv.z), -1, -1, -1, rec, o);
+            rc = region_plan<MODE, RL>(d, sh, l, gm, g0, p, make_int2(mv.y, mv.z), -1, -1, -1, rec, o);
         } else {
             const int inst = B.ninst > 1 ? csr_find(B.pofs, B.ninst + 1, item) : 0;
             const int p0 = __ldg(B.pofs + inst), j = item - p0;
@@ -200,7 +201,7 @@ __global__ void __launch_bounds__(ROUND_THREADS, ROUND_BLOCKS) k_round_plan(Dev 
                 a &= a - 1;
                 start = __ldcg(d.pt_tri + __ldg(B.order + p0 + a));
             }
-            rc = region_plan<false, RL>(d, sh, l, gm, g0, p, q, start, s, s + 1, rec, o);
+            rc = region_plan<REGION_INSERT, RL>(d, sh, l, gm, g0, p, q, start, s, s + 1, rec, o);
         }
         ex += o.ex;
         ti += o.ti;
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(ROUND_THREADS, ROUND_BLOCKS) k_round_plan(Dev 
         if (l == 0) {
             steps += o.steps;
             if (nt < 0) R.left[atomicAdd(R.left_count, 1)] = item;
-            R.hdr[x] = make_int4(item, nt, pr, o.k | o.ncav << 8 | o.edge << 24 | o.ghost << 25);
+            R.hdr[x] = make_int4(item, nt, pr, o.k | o.ncav << 8 | o.edge << 24 | o.ghost << 25 | o.prop << 26);
         }
         __syncwarp(gm);
     }
@@ -244,7 +245,7 @@ __global__ void __launch_bounds__(256) k_round_commit(Dev d, Rounds R, int b, Ro
     round_window(R, b, total, nlost, head, count);
     const int lane = threadIdx.x & (ROUND_LANES - 1);
     const unsigned gm = 0xffu << (threadIdx.x & 24);  // this operation's lanes
-    int nwin = 0, nlose = 0, degs = 0, flips = 0, edges = 0, ghosts = 0;
+    int nwin = 0, nlose = 0, degs = 0, flips = 0, edges = 0, ghosts = 0, props = 0, hits = 0;
     const int groups = gridDim.x * (blockDim.x / ROUND_LANES);
     // (whole warps take part in the ballots: the loop ends for a warp at once)
     for (int x0 = (blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / ROUND_LANES; x0 < count; x0 += groups) {
@@ -295,6 +296,8 @@ __global__ void __launch_bounds__(256) k_round_commit(Dev d, Rounds R, int b, Ro
                 flips += ((h.w >> 8) & 0xffff) - 1;
                 edges += (h.w >> 24) & 1;
                 ghosts += (h.w >> 25) & 1;
+                props += (h.w >> 26) & 1;
+                hits += (h.w >> 27) & 1;
             } else {
                 ++nlose;
                 R.lost[(b + 1) & 1][atomicAdd(R.lostcnt + b + 1, 1)] = h.x;
@@ -302,19 +305,20 @@ __global__ void __launch_bounds__(256) k_round_commit(Dev d, Rounds R, int b, Ro
         }
     }
     if (!d.counters) return;
-    __shared__ int sum[6];
-    if (threadIdx.x < 6) sum[threadIdx.x] = 0;
+    __shared__ int sum[8];
+    if (threadIdx.x < 8) sum[threadIdx.x] = 0;
     __syncthreads();
-    const int part[6] = {nwin, nlose, degs, flips, edges, ghosts};
+    const int part[8] = {nwin, nlose, degs, flips, edges, ghosts, props, hits};
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
+    for (int i = 0; i < 8; ++i) {
         const int s = __reduce_add_sync(FULL, part[i]);
         if ((threadIdx.x & 31) == 0 && s) atomicAdd(sum + i, s);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        const int slot[6] = {C_INSERTS, C_RETRIES, C_DEG_DEL, C_FLIPS, C_SPLIT_EDGE, C_SPLIT_GHOST};
-        for (int i = 0; i < 6; ++i)
+        const int slot[8] = {C_INSERTS,    C_RETRIES,     C_DEG_DEL,    C_FLIPS,
+                             C_SPLIT_EDGE, C_SPLIT_GHOST, C_PROP_MOVES, C_PROP_HITS};
+        for (int i = 0; i < 8; ++i)
             if (sum[i]) atomicAdd(d.counters + slot[i], (unsigned long long)sum[i]);
         if (MOVE && sum[0]) atomicAdd(d.counters + C_DELETES, (unsigned long long)sum[0]);
     }
