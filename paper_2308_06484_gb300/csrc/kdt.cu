@@ -1430,11 +1430,14 @@ int export_range(kdt *h, int s0, int nslots, int idbase, int np, int32_t *out, i
     cudaStream_t st = h->stream;
     int s = 4;
     while (s < EXB_SHIFT && (np >> s) > 2048) ++s;
+    int bits = 1;
+    while ((np - 1) >> bits) ++bits;
+    s = std::min(s, 64 - 2 * bits);  // (a row is one word; 8 for 2^28 points)
     const int nb = ((np - 1) >> s) + 1;
     const bool dev_out = cap > 0 && on_device(h, out);
     const int64_t room = std::min<int64_t>(cap, 2 * (int64_t)np);  // (2 np - 5 rows at most)
     if (grow(h->exp_cnt, ((size_t)(EXB_PAD + 1) * nb + 1) * sizeof(int)) ||
-        (cap > 0 && grow(h->exp_rows, (size_t)std::max<int64_t>(room, 1) * sizeof(int3))) ||
+        (cap > 0 && grow(h->exp_rows, (size_t)std::max<int64_t>(room, 1) * sizeof(unsigned long long))) ||
         (cap > 0 && !dev_out && grow(h->exp_out, (size_t)room * sizeof(int3))))
         return KDT_ERR_CUDA;
     int *cnt = (int *)h->exp_cnt.p, *off = cnt + (size_t)EXB_PAD * nb;
@@ -1446,10 +1449,10 @@ int export_range(kdt *h, int s0, int nslots, int idbase, int np, int32_t *out, i
     h->stats.kernel_launches += 2;
     int32_t *dst = dev_out ? out : (int32_t *)h->exp_out.p;
     if (cap > 0) {
-        const size_t smem = ((2 + 3 * (size_t)EXB_ROWS) << s) * sizeof(int);
-        k_exb_append<<<thread_grid(h, nslots, 256), 256, 0, st>>>(tv, nslots, cnt, (int3 *)h->exp_rows.p, idbase, s, total,
-                                                                 most, cap);
-        k_exb_sort<<<nb, EXB_THREADS, smem, st>>>((const int3 *)h->exp_rows.p, off, s, dst, total, most, cap);
+        const size_t smem = ((2 + 2 * (size_t)EXB_ROWS) << s) * sizeof(int);
+        unsigned long long *rows = (unsigned long long *)h->exp_rows.p;
+        k_exb_append<<<thread_grid(h, nslots, 256), 256, 0, st>>>(tv, nslots, cnt, rows, idbase, s, bits, total, most, cap);
+        k_exb_sort<<<nb, EXB_THREADS, smem, st>>>(rows, off, s, bits, dst, total, most, cap);
         h->stats.kernel_launches += 2;
     }
     CK(cudaGetLastError());
@@ -1665,7 +1668,7 @@ int kdt_create(kdt **out, const kdt_config *cfg, int device, void *cuda_stream)
         cudaFuncSetAttribute(k_mlp_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TCS_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_mlp_grad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TG_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_exb_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(((2 + 3 * EXB_ROWS) << EXB_SHIFT) * sizeof(int))) != cudaSuccess) {
+                             (int)(((2 + 2 * EXB_ROWS) << EXB_SHIFT) * sizeof(int))) != cudaSuccess) {
         kdt_destroy(h);
         return KDT_ERR_CUDA;
     }

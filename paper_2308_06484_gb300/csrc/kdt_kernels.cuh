@@ -1149,7 +1149,7 @@ __global__ void k_exp_sortseg(int n, const int *off, const int *cnt, int3 *out)
 // 1.45), 1.67 ms in buckets; 512 instances, 21.7e6 points: 3.24 -> 2.04; 1e6 points: 215 ->
 // 175 us; 1,000 points: 80 -> 48 us (four launches and one wait instead of eight and two).
 constexpr int EXB_ROWS = 7;     // rows a bucket may hold per first id (mean 2, up to 6 at the lowest ids)
-constexpr int EXB_SHIFT = 9;    // largest s: 43 KB of rows a block, five blocks per SM
+constexpr int EXB_SHIFT = 9;    // largest s: 33 KB a block
 constexpr int EXB_THREADS = 256;
 constexpr int EXB_PAD = 8;      // ints between two buckets' counters: a sector each, or the atomics of many
                                 // buckets queue at one
@@ -1209,42 +1209,52 @@ __global__ void __launch_bounds__(1024) k_exb_scan(int *cnt, int nb, int *off, i
     if (threadIdx.x == 1023) off[nb] = run;
 }
 
-// every row (smallest id first, local ids) to the end of its bucket; nothing when the list
-// does not fit the caller's room or a bucket its block
-__global__ void k_exb_append(TriHalf tv, int nslots, int *cur, int3 *rows, int idbase, int s, const int *total,
-                             const int *most, long long cap)
+// Every row (smallest id first, local ids) to the end of its bucket, packed into one word:
+// the first id's place in the bucket, then the other two ids of `bits` bits each.  (One
+// 8-byte store a row: three 4-byte stores of a row cost three sector writes in L2.)
+// Nothing when the list does not fit the caller's room or a bucket its block.
+__global__ void k_exb_append(TriHalf tv, int nslots, int *cur, unsigned long long *rows, int idbase, int s, int bits,
+                             const int *total, const int *most, long long cap)
 {
     if (__ldcg(total) > cap || __ldcg(most) > EXB_ROWS << s) return;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nslots; t += gridDim.x * blockDim.x) {
         const int4 v = __ldcg(tv + t);
         if (!finite_alive(v)) continue;
-        int3 r;
-        if (v.x < v.y && v.x < v.z) r = make_int3(v.x, v.y, v.z);
-        else if (v.y < v.z) r = make_int3(v.y, v.z, v.x);
-        else r = make_int3(v.z, v.x, v.y);
-        r.x -= idbase;
-        r.y -= idbase;
-        r.z -= idbase;
-        rows[atomicAdd(cur + (r.x >> s) * EXB_PAD, 1)] = r;
+        int a = v.x, b = v.y, c = v.z;
+        if (v.y < v.x && v.y < v.z) {
+            a = v.y;
+            b = v.z;
+            c = v.x;
+        } else if (v.z < v.x && v.z < v.y) {
+            a = v.z;
+            b = v.x;
+            c = v.y;
+        }
+        a -= idbase;
+        rows[atomicAdd(cur + (a >> s) * EXB_PAD, 1)] =
+            (unsigned long long)(a & ((1 << s) - 1)) << 2 * bits | (unsigned long long)(b - idbase) << bits |
+            (unsigned long long)(c - idbase);
     }
 }
 
-// One block per bucket: counting sort by the first id in shared memory, each first id's rows
-// by the second (which differs from row to row: one triangle left of every edge a -> b),
-// then the bucket in one piece.
-__global__ void __launch_bounds__(EXB_THREADS) k_exb_sort(const int3 *rows, const int *off, int s, int *out,
-                                                          const int *total, const int *most, long long cap)
+// One block per bucket: counting sort by the first id in shared memory, each first id's
+// rows as words (the second ids of one first id's rows differ: one triangle left of every
+// edge a -> b), then the bucket in one piece.
+__global__ void __launch_bounds__(EXB_THREADS) k_exb_sort(const unsigned long long *rows, const int *off, int s,
+                                                          int bits, int *out, const int *total, const int *most,
+                                                          long long cap)
 {
     if (__ldcg(total) > cap || __ldcg(most) > EXB_ROWS << s) return;
-    extern __shared__ int exb[];
+    extern __shared__ unsigned long long exb[];
     const int ids = 1 << s, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int *start = exb, *fill = exb + ids, *r = exb + 2 * ids;  // (r: three ints a row)
+    unsigned long long *r = exb;
+    int *start = reinterpret_cast<int *>(exb + (EXB_ROWS << s)), *fill = start + ids;
     __shared__ int ws[EXB_THREADS / 32];
     const int base = off[blockIdx.x], n = off[blockIdx.x + 1] - base;
     for (int i = threadIdx.x; i < ids; i += EXB_THREADS) fill[i] = 0;
     __syncthreads();
-    const int *in = reinterpret_cast<const int *>(rows + base);
-    for (int i = threadIdx.x; i < n; i += EXB_THREADS) atomicAdd(fill + (__ldg(in + 3 * i) & (ids - 1)), 1);
+    const unsigned long long *in = rows + base;
+    for (int i = threadIdx.x; i < n; i += EXB_THREADS) atomicAdd(fill + (int)(__ldg(in + i) >> 2 * bits), 1);
     __syncthreads();
     // exclusive scan of the counts, `per` ids a thread
     const int per = (ids + EXB_THREADS - 1) / EXB_THREADS, lo = min(ids, (int)threadIdx.x * per), hi = min(ids, lo + per);
@@ -1267,28 +1277,27 @@ __global__ void __launch_bounds__(EXB_THREADS) k_exb_sort(const int3 *rows, cons
     }
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += EXB_THREADS) {
-        const int a = __ldg(in + 3 * i), b = __ldg(in + 3 * i + 1), c = __ldg(in + 3 * i + 2);
-        const int at = 3 * atomicAdd(fill + (a & (ids - 1)), 1);
-        r[at] = a;
-        r[at + 1] = b;
-        r[at + 2] = c;
+        const unsigned long long w = __ldg(in + i);
+        r[atomicAdd(fill + (int)(w >> 2 * bits), 1)] = w;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < ids; i += EXB_THREADS) {
         const int b0 = start[i], e0 = fill[i];
         for (int j = b0 + 1; j < e0; ++j) {
-            const int y = r[3 * j + 1], z = r[3 * j + 2];
+            const unsigned long long w = r[j];
             int k = j - 1;
-            for (; k >= b0 && r[3 * k + 1] > y; --k) {
-                r[3 * k + 4] = r[3 * k + 1];
-                r[3 * k + 5] = r[3 * k + 2];
-            }
-            r[3 * k + 4] = y;
-            r[3 * k + 5] = z;
+            for (; k >= b0 && r[k] > w; --k) r[k + 1] = r[k];
+            r[k + 1] = w;
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < 3 * n; i += EXB_THREADS) out[3ll * base + i] = r[i];
+    const unsigned long long mask = (1ull << bits) - 1ull;
+    const int a0 = (int)blockIdx.x << s;
+    for (int i = threadIdx.x; i < 3 * n; i += EXB_THREADS) {
+        const int j = i / 3, f = i - 3 * j;
+        const unsigned long long w = r[j];
+        out[3ll * base + i] = f == 0 ? a0 + (int)(w >> 2 * bits) : (f == 1 ? (int)((w >> bits) & mask) : (int)(w & mask));
+    }
 }
 
 // ------------------------------------------------------------------ verifier
