@@ -51,6 +51,9 @@ struct kdt {
     kdt_config cfg{};
     int64_t n = 0;  // points (all instances)
     int cap = 0;    // triangle slots (all instances)
+    // room of the state's arrays: a build of as many points or somewhat fewer keeps them
+    int64_t n_room = 0, cells_room = 0;
+    int inst_room = 0;
     bool built = false;
     bool order_valid = false;  // bord holds every point, in the last build's Hilbert order
     int stamp = 0;
@@ -93,6 +96,7 @@ struct kdt {
     Buf rb_cnt, rb_lost, rb_hdr, rb_rec, rb_queue, rb_left;
     Buf rm_cnt, rm_lost, rm_hdr, rm_rec, rm_slots, rm_left;
     int rm_rounds = 0, rm_ops = 0;
+    int rm_layout = 0;  // rounds the counters have room for (a small step's too)
     // d-calculation: results, running minimum (per N)
     Buf dc_dist, dc_cmin, dc_scal;
     int64_t d2_run = INT64_MAX;
@@ -124,9 +128,11 @@ struct kdt {
     int *ctl = nullptr;   // device
     int *hctl = nullptr;  // pinned host
     cudaStream_t cstream = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t gexec = nullptr;
-    int graph_gen = -1;  // buffer generation the graph was captured for
+    // [0]: the step's graph, [1]: a small step's (k_step_small), and the buffer generation
+    // each was captured for
+    cudaGraph_t graph[2] = {nullptr, nullptr};
+    cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+    int graph_gen[2] = {-1, -1};
     int gen = 0;         // bumped whenever step buffers or tables change
     // autotuner state: configuration index being timed, accumulated times
     int tune_idx = -1;
@@ -286,6 +292,8 @@ Inst make_inst(kdt *h)
     I.stride = h->cfg.partition_order == 0 && !h->qhist ? h->stride : 1;
     I.ncells_dyn = h->qhist ? h->scal + S_NCELLS : nullptr;
     I.pending = nullptr;
+    I.left = nullptr;
+    I.few_left = 0;
     return I;
 }
 
@@ -553,7 +561,7 @@ int rebuild_instance(kdt *h, int i)
     CK(cudaMemcpyAsync(h->scal + S_THIRD, &third0, sizeof(int), cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(h->tri + 2 * (size_t)s0, 0, 2 * (size_t)capi * sizeof(int4), st));
     k_fill_int<<<thread_grid(h, n, 256), 256, 0, st>>>(h->pt_tri + p0, n, -1);
-    k_range<<<thread_grid(h, n, 256), 256, 0, st>>>(h->xy + p0, n, h->cfg.domain_bits, h->scal + S_STATUS,
+    k_range<<<std::min(thread_grid(h, n, 256), 4 * sm_count(h->device)), 256, 0, st>>>(h->xy + p0, n, h->cfg.domain_bits, h->scal + S_STATUS,
                                                     h->scal + S_MINX);
     h->stats.kernel_launches += 2;
     if (sync_scalars(h)) return KDT_ERR_CUDA;
@@ -624,7 +632,7 @@ int rebuild_batch(kdt *h)
     CK(cudaMemcpyAsync(bbox, hb.data(), hb.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(h->tri, 0, 2 * (size_t)h->cap * sizeof(int4), st));
     k_fill_int<<<thread_grid(h, n, 256), 256, 0, st>>>(h->pt_tri, n, -1);
-    k_range_batch<<<thread_grid(h, n, 256), 256, 0, st>>>(h->xy, n, h->d_pofs, ni, h->cfg.domain_bits,
+    k_range_batch<<<thread_grid(h, (n + 31) / 32, 256), 256, 0, st>>>(h->xy, n, h->d_pofs, ni, h->cfg.domain_bits,
                                                           h->scal + S_STATUS, bbox);
     h->stats.kernel_launches += 2;
     CK(cudaMemcpyAsync(hb.data(), bbox, hb.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -737,6 +745,7 @@ int ensure_moves(kdt *h, int64_t m)
 // An empty round costs about 5 us (4 more on 1e6 points: 85 -> 120 us a step), a round more
 // on 16e6 clustered points saves 30 us (2 rounds 1.55, 4 1.47, 6 1.43 ms), on 512 instances
 // it costs 20.
+constexpr int FEW_LEFT = 1024;  // moves the kinetic kernel takes as a list, a warp each
 constexpr int STEP_EXTRA_ROUNDS = 2, STEP_EXTRA_ROUNDS_MANY = 4, STEP_MANY = 32768;
 
 // Do the step's moves go through rounds?  The paper's method (delete and insert), without
@@ -754,12 +763,14 @@ int ensure_rounds(kdt *h)
     const int ops = std::min(h->mcap, ROUND_OPS);
     const int rounds =
         (h->mcap + ops - 1) / ops + (h->mcap >= STEP_MANY ? STEP_EXTRA_ROUNDS_MANY : STEP_EXTRA_ROUNDS);
-    if (grow(h->rm_cnt, round_counter_ints(rounds) * sizeof(int)) || grow(h->rm_lost, 2 * (size_t)ops * sizeof(int)) ||
+    const int layout = std::max(rounds, SMALL_ROUNDS);
+    if (grow(h->rm_cnt, round_counter_ints(layout) * sizeof(int)) || grow(h->rm_lost, 2 * (size_t)ops * sizeof(int)) ||
         grow(h->rm_hdr, (size_t)ops * sizeof(int4)) || grow(h->rm_rec, (size_t)ops * 2 * RT * sizeof(int4)) ||
-        grow(h->rm_slots, (size_t)rounds * ops * RT * sizeof(int)) || grow(h->rm_left, (size_t)h->mcap * sizeof(int)))
+        grow(h->rm_slots, std::max((size_t)rounds * ops, (size_t)SMALL_ROUNDS * SMALL_MOVES) * RT * sizeof(int)) || grow(h->rm_left, (size_t)h->mcap * sizeof(int)))
         return KDT_ERR_CUDA;
     h->rm_ops = ops;
     h->rm_rounds = rounds;
+    h->rm_layout = layout;
     h->gen++;
     return 0;
 }
@@ -801,35 +812,71 @@ int set_partitions(kdt *h, int ppp)
     // a quad-tree re-divided at every step has at most one leaf per fine cell
     const long long cap = h->qhist ? (long long)h->qF * h->qF : cells;
     h->ncells_cap = (int)cap;
-    if (dalloc(&h->head, (size_t)cap) || dalloc(&h->d_cofs, h->ninst + 1) || dalloc(&h->d_grid, h->ninst) ||
-        dalloc(&h->dloc2, (size_t)cap) || dalloc(&h->pcost, (size_t)cap) || dalloc(&h->order, (size_t)cap))
-        return KDT_ERR_CUDA;
+    if (cap > h->cells_room) {
+        h->cells_room = 0;
+        if (dalloc(&h->head, (size_t)cap) || dalloc(&h->dloc2, (size_t)cap) || dalloc(&h->pcost, (size_t)cap) ||
+            dalloc(&h->order, (size_t)cap))
+            return KDT_ERR_CUDA;
+        h->cells_room = cap;
+    }
     k_fill_u64<<<thread_grid(h, cap, 256), 256, 0, h->stream>>>(h->dloc2, cap, (unsigned long long)INT64_MAX);
     h->stats.kernel_launches++;
     h->dloc_valid = false;
-    CK(cudaMemcpy(h->d_cofs, h->cofs.data(), (h->ninst + 1) * sizeof(int), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(h->d_grid, h->igrid.data(), h->ninst * sizeof(int), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(h->d_cofs, h->cofs.data(), (h->ninst + 1) * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+    CK(cudaMemcpyAsync(h->d_grid, h->igrid.data(), h->ninst * sizeof(int), cudaMemcpyHostToDevice, h->stream));
     h->gen++;
     return 0;
 }
 
-void drop_graph(kdt *h)
+void drop_graph(kdt *h, int which)
 {
-    if (h->gexec) cudaGraphExecDestroy(h->gexec);
-    if (h->graph) cudaGraphDestroy(h->graph);
-    h->gexec = nullptr;
-    h->graph = nullptr;
-    h->graph_gen = -1;
+    if (h->gexec[which]) cudaGraphExecDestroy(h->gexec[which]);
+    if (h->graph[which]) cudaGraphDestroy(h->graph[which]);
+    h->gexec[which] = nullptr;
+    h->graph[which] = nullptr;
+    h->graph_gen[which] = -1;
+}
+
+void free_quadtree(kdt *h)
+{
+    void *ps[] = {h->qmap, h->qhist, h->qpyr, h->qflag, h->qpre, h->qlev};
+    for (void *p : ps)
+        if (p) cudaFree(p);
+    h->qmap = nullptr;
+    h->qhist = nullptr;
+    h->qpyr = nullptr;
+    h->qflag = nullptr;
+    h->qpre = nullptr;
+    h->qlev = nullptr;
+    h->qleaves = 0;
+}
+
+// No triangulation any more, the arrays kept for the next build.
+void reset_state(kdt *h)
+{
+    drop_graph(h, 0);
+    drop_graph(h, 1);
+    h->gen++;
+    free_quadtree(h);
+    h->dloc_valid = false;
+    h->order_valid = false;
+    h->n = 0;
+    h->cap = 0;
+    h->ninst = 0;
+    h->built = false;
+    h->tune_idx = -1;
+    h->tune_done = 0;
 }
 
 void free_state(kdt *h)
 {
-    drop_graph(h);
-    h->gen++;
+    reset_state(h);
+    h->n_room = 0;
+    h->cells_room = 0;
+    h->inst_room = 0;
     void *ps[] = {h->xy, h->pt_tri, h->pt_stamp, h->tri, h->viol, h->moves, h->gmoves, h->old_xy,
                   h->next, h->head, h->deferred, h->dirty, h->scan_tmp, h->d_pofs, h->d_cofs, h->d_grid,
-                  h->ctl, h->d_tofs, h->qmap, h->dloc2, h->pcost, h->order, h->ohist, h->pguess,
-                  h->qhist, h->qpyr, h->qflag, h->qpre, h->qlev, h->pfeat, h->ppart};
+                  h->ctl, h->d_tofs, h->dloc2, h->pcost, h->order, h->ohist, h->pguess, h->pfeat, h->ppart};
     for (void *p : ps)
         if (p) cudaFree(p);
     if (h->hctl) cudaFreeHost(h->hctl);
@@ -840,34 +887,19 @@ void free_state(kdt *h)
     h->head = nullptr; h->deferred = nullptr; h->dirty = nullptr; h->scan_tmp = nullptr;
     h->d_pofs = nullptr; h->d_cofs = nullptr; h->d_grid = nullptr; h->d_moff = nullptr; h->h_moff = nullptr;
     h->d_tofs = nullptr;
-    h->qmap = nullptr;
-    h->qhist = nullptr;
-    h->qpyr = nullptr;
-    h->qflag = nullptr;
-    h->qpre = nullptr;
-    h->qlev = nullptr;
     h->dloc2 = nullptr;
-    h->dloc_valid = false;
     h->pcost = nullptr;
     h->order = nullptr;
     h->ohist = nullptr;
     h->pguess = nullptr;
     h->pfeat = nullptr;
     h->ppart = nullptr;
-    h->qleaves = 0;
     h->mcap = 0; h->dirty_cap = 0; h->scan_tmp_cap = 0; h->rm_rounds = 0;
     Buf *bs[] = {&h->key, &h->bord, &h->hist, &h->hoff, &h->exp_cnt, &h->exp_off, &h->exp_fill, &h->exp_out, &h->exp_rows,
                  &h->btab, &h->blev, &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left,
                  &h->rm_cnt, &h->rm_lost, &h->rm_hdr, &h->rm_rec, &h->rm_slots, &h->rm_left,
                  &h->dc_dist, &h->dc_cmin, &h->dc_scal};
     for (Buf *b : bs) free_buf(*b);
-    h->n = 0;
-    h->cap = 0;
-    h->ninst = 0;
-    h->built = false;
-    h->order_valid = false;
-    h->tune_idx = -1;
-    h->tune_done = 0;
 }
 
 // state for instances with point offsets `offs` (host, n_inst + 1 entries)
@@ -883,17 +915,30 @@ int alloc_state(kdt *h, const int64_t *offs, int n_inst)
     h->n = offs[n_inst];
     h->cap = h->tofs[n_inst];
     h->built = false;
-    if (dalloc(&h->xy, h->n) || dalloc(&h->pt_tri, h->n) || dalloc(&h->pt_stamp, h->n) || dalloc(&h->tri, 2 * (size_t)h->cap) || dalloc(&h->d_pofs, n_inst + 1) || dalloc(&h->ctl, 4 + n_inst + 1) ||
-        dalloc(&h->d_tofs, n_inst + 1) || dalloc(&h->pguess, h->n) || dalloc(&h->ohist, 2 * PLAN_CLASSES))
-        return KDT_ERR_CUDA;
-    if (cudaMallocHost(&h->hctl, (4 + n_inst + 1) * sizeof(int)) != cudaSuccess) return KDT_ERR_CUDA;
+    if (h->n > h->n_room) {
+        h->n_room = 0;
+        if (dalloc(&h->xy, h->n) || dalloc(&h->pt_tri, h->n) || dalloc(&h->pt_stamp, h->n) ||
+            dalloc(&h->tri, 4 * (size_t)h->n) || dalloc(&h->pguess, h->n) ||
+            dalloc(&h->viol, std::max<size_t>(4096, 2 * (size_t)h->n)))
+            return KDT_ERR_CUDA;
+        h->n_room = h->n;
+    }
+    if (n_inst > h->inst_room) {
+        h->inst_room = 0;
+        if (h->hctl) cudaFreeHost(h->hctl);
+        h->hctl = nullptr;
+        if (dalloc(&h->d_pofs, n_inst + 1) || dalloc(&h->ctl, 4 + n_inst + 1) || dalloc(&h->d_tofs, n_inst + 1) ||
+            dalloc(&h->d_cofs, n_inst + 1) || dalloc(&h->d_grid, n_inst) || dalloc(&h->ohist, 2 * PLAN_CLASSES) ||
+            cudaMallocHost(&h->hctl, (4 + n_inst + 1) * sizeof(int)) != cudaSuccess)
+            return KDT_ERR_CUDA;
+        h->inst_room = n_inst;
+    }
     h->d_moff = h->ctl + 4;
     h->h_moff = h->hctl + 4;
-    CK(cudaMemcpy(h->d_pofs, h->pofs.data(), (n_inst + 1) * sizeof(int), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(h->d_tofs, h->tofs.data(), (n_inst + 1) * sizeof(int), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(h->d_pofs, h->pofs.data(), (n_inst + 1) * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+    CK(cudaMemcpyAsync(h->d_tofs, h->tofs.data(), (n_inst + 1) * sizeof(int), cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemsetAsync(h->pt_stamp, 0, h->n * sizeof(int), h->stream));
     h->viol_cap = std::max(4096, h->cap);
-    if (dalloc(&h->viol, (size_t)h->viol_cap)) return KDT_ERR_CUDA;
     int ppp = h->cfg.points_per_partition > 0 ? h->cfg.points_per_partition : 256;
     h->wpp = h->cfg.warps_per_partition > 0 ? h->cfg.warps_per_partition : 1;
     h->tune_idx = h->cfg.autotune ? 0 : -1;
@@ -983,6 +1028,27 @@ int verify_state(kdt *h, int64_t *bad)
     return 0;
 }
 
+void kinetic_shape(kdt *h, int *blocks, int *threads);
+
+// The kinetic kernel, the certification of its global-path writes, the status to the host.
+int enqueue_kinetic(kdt *h, cudaStream_t st, const Dev &d, const Inst &I, bool from_ctl, int defer_cap)
+{
+    // inside a capture an event record must be an external node to keep its timestamp
+    const unsigned evflags = from_ctl ? cudaEventRecordExternal : cudaEventRecordDefault;
+    int kblocks = 0, kthreads = 0;
+    kinetic_shape(h, &kblocks, &kthreads);
+    Dev dk = d;
+    dk.big = h->big;
+    auto kin = h->cfg.kinetic_blocks_per_sm == 7 ? k_kinetic<7> : k_kinetic<6>;
+    kin<<<kblocks, kthreads, 0, st>>>(dk, h->gmoves, h->head, h->next, I, h->ncells, h->wpp, h->deferred,
+                                      h->scal + S_DEFER, defer_cap, h->viol, h->viol_cap);
+    if (h->cfg.timing) CK(cudaEventRecordWithFlags(h->ev1, st, evflags));
+    k_certify_step<<<thread_grid(h, 4096, 256), 256, 0, st>>>(d, h->viol, h->scal + S_VIOL, h->viol_cap);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(h->hscal, h->scal, S_NUM * sizeof(int), cudaMemcpyDeviceToHost, st));
+    return 0;
+}
+
 // Issue one step's kernels on `st`: intake + per-partition lists, the kinetic kernel
 // (whose last warp inserts deferred points and certifies global-path writes), and the
 // copy of the status scalars to the host.  With from_ctl the kernels read m, the
@@ -1036,7 +1102,7 @@ int tc_grid(const kdt *h, long long rows)
     return (int)std::min<long long>(tiles, 3ll * sm_count(h->device));
 }
 
-int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, bool from_ctl)
+int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, bool from_ctl, bool small)
 {
     int cap = from_ctl ? h->mcap : mi;
     Inst I = make_inst(h);
@@ -1044,10 +1110,29 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
     // copy reads them when the graph runs)
     CK(cudaMemcpyAsync(h->ctl, h->hctl, (4 + h->ninst + 1) * sizeof(int), cudaMemcpyHostToDevice, st));
     const bool rounds = step_in_rounds(h);
+    const unsigned evflags0 = from_ctl ? cudaEventRecordExternal : cudaEventRecordDefault;
+    Rounds R{};
+    if (rounds) {
+        R = make_rounds(h->rm_cnt, h->rm_layout, h->rm_lost, h->rm_hdr, h->rm_rec, h->rm_ops);
+        R.slots = (int *)h->rm_slots.p;
+        R.left = (int *)h->rm_left.p;
+        I.pending = R.pending;
+        I.left = R.left;
+        I.few_left = std::min(FEW_LEFT, h->mcap / 4);  // (each can be left for later DQ_PASSES times)
+    }
+    if (small) {
+        if (h->cfg.timing) CK(cudaEventRecordWithFlags(h->ev0, st, evflags0));
+        // (a small step's moves push a few entries each onto the deferred list)
+        const int ndef = std::min(h->mcap, 8 * SMALL_MOVES);
+        k_step_small<<<1, SMALL_THREADS, 0, st>>>(d, mp, mi, I, h->cfg.domain_bits, h->scal, S_NUM, h->head, h->ncells_cap,
+                                                  h->next, h->deferred, ndef, h->old_xy, h->gmoves, h->dloc2, far2(h), R,
+                                                  (int *)h->rm_cnt.p, (int)round_counter_ints(h->rm_layout));
+        return enqueue_kinetic(h, st, d, I, from_ctl, ndef);
+    }
     // scalars zero, partition lists empty, deferred entries -1: one kernel
     k_step_clear<<<thread_grid(h, std::max<long long>(h->ncells_cap, 4ll * h->mcap), 256), 256, 0, st>>>(
         h->scal, S_NUM, h->head, h->ncells_cap, h->deferred, h->mcap,
-        rounds ? (int *)h->rm_cnt.p : nullptr, rounds ? (int)round_counter_ints(h->rm_rounds) : 0);
+        rounds ? (int *)h->rm_cnt.p : nullptr, rounds ? (int)round_counter_ints(h->rm_layout) : 0);
     if (h->qhist) {
         // Fig. 4's Quad-treeDvision at the start of the step, from the points per fine
         // cell the intakes keep current: count pyramid, every fine cell's leaf, leaves
@@ -1093,35 +1178,18 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
         k_order<<<thread_grid(h, h->ncells_cap, 256), 256, 0, st>>>(h->pcost, h->ncells_cap, h->ohist, h->order, 1,
                                                                     ostride);
     }
-    // inside a capture an event record must be an external node to keep its timestamp
-    unsigned evflags = from_ctl ? cudaEventRecordExternal : cudaEventRecordDefault;
-    if (h->cfg.timing) CK(cudaEventRecordWithFlags(h->ev0, st, evflags));
+    if (h->cfg.timing) CK(cudaEventRecordWithFlags(h->ev0, st, evflags0));
     if (rounds) {
-        Rounds R = make_rounds(h->rm_cnt, h->rm_rounds, h->rm_lost, h->rm_hdr, h->rm_rec, h->rm_ops);
-        R.slots = (int *)h->rm_slots.p;
-        R.left = (int *)h->rm_left.p;
         const RoundMoves M{h->gmoves};
         const RoundBuild B{nullptr, nullptr, nullptr, nullptr, nullptr, 0, mi, 0};
         auto launch_moves = d.pguess ? launch_round<REGION_GUESS> : launch_round<REGION_MOVE>;
         for (int b = 0; b < h->rm_rounds; ++b)
             launch_moves(h, st, d, R, b, std::min(cap, h->rm_ops), M, B, b + 1 == h->rm_rounds,
-                               b + 1 == h->rm_rounds);
+                         b + 1 == h->rm_rounds);
         k_round_clear<<<thread_grid(h, (long long)cap * (RT / 4), 256), 256, 0, st>>>(
             d, R, h->rm_rounds, mi, I, h->cfg.domain_bits, h->gmoves, h->old_xy, h->head, h->next);
-        I.pending = R.pending;
     }
-    int kblocks = 0, kthreads = 0;
-    kinetic_shape(h, &kblocks, &kthreads);
-    Dev dk = d;
-    dk.big = h->big;
-    auto kin = h->cfg.kinetic_blocks_per_sm == 7 ? k_kinetic<7> : k_kinetic<6>;
-    kin<<<kblocks, kthreads, 0, st>>>(dk, h->gmoves, h->head, h->next, I, h->ncells, h->wpp, h->deferred,
-                                            h->scal + S_DEFER, h->mcap, h->viol, h->viol_cap);
-    if (h->cfg.timing) CK(cudaEventRecordWithFlags(h->ev1, st, evflags));
-    k_certify_step<<<thread_grid(h, 4096, 256), 256, 0, st>>>(d, h->viol, h->scal + S_VIOL, h->viol_cap);
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(h->hscal, h->scal, S_NUM * sizeof(int), cudaMemcpyDeviceToHost, st));
-    return 0;
+    return enqueue_kinetic(h, st, d, I, from_ctl, h->mcap);
 }
 
 // After the step kernels: repair the violations they recorded (general Lawson) and
@@ -1283,23 +1351,26 @@ int step_core(kdt *h, const kdt_move *moves, const int64_t *moff, int64_t m)
     }
     d = make_dev(h);
     bool timed = h->cfg.timing || (h->tune_idx >= 0 && !h->tune_done);
+    const bool rounds = step_in_rounds(h);
+    const bool small = rounds && m <= SMALL_MOVES && h->cfg.plan == 0 && !h->qhist && h->ncells_cap <= SMALL_CELLS;
+    const int which = small ? 1 : 0;
     if (h->cfg.use_graph) {
         // one graph launch per step
-        if (h->graph_gen != h->gen) {
-            drop_graph(h);
+        if (h->graph_gen[which] != h->gen) {
+            drop_graph(h, which);
             Dev dg = d;
             dg.ctl = h->ctl;
             CK(cudaStreamBeginCapture(h->cstream, cudaStreamCaptureModeThreadLocal));
-            int er = enqueue_step(h, h->cstream, dg, nullptr, 0, true);
+            int er = enqueue_step(h, h->cstream, dg, nullptr, 0, true, small);
             cudaGraph_t g = nullptr;
             cudaError_t ce = cudaStreamEndCapture(h->cstream, &g);
             if (er || ce != cudaSuccess) {
                 if (g) cudaGraphDestroy(g);
                 return KDT_ERR_CUDA;
             }
-            h->graph = g;
-            CK(cudaGraphInstantiate(&h->gexec, h->graph, 0));
-            h->graph_gen = h->gen;
+            h->graph[which] = g;
+            CK(cudaGraphInstantiate(&h->gexec[which], h->graph[which], 0));
+            h->graph_gen[which] = h->gen;
         }
         h->hctl[0] = mi;
         h->hctl[1] = h->stamp;
@@ -1307,17 +1378,17 @@ int step_core(kdt *h, const kdt_move *moves, const int64_t *moff, int64_t m)
         h->hctl[2] = (int)(unsigned)(pa & 0xffffffffu);
         h->hctl[3] = (int)(unsigned)(pa >> 32);
         if (timed) CK(cudaEventRecord(h->ev2, st));
-        CK(cudaGraphLaunch(h->gexec, st));
+        CK(cudaGraphLaunch(h->gexec[which], st));
         if (timed) CK(cudaEventRecord(h->ev3, st));
     } else {
         if (timed) CK(cudaEventRecord(h->ev2, st));
-        if (enqueue_step(h, st, d, mp, mi, false)) return KDT_ERR_CUDA;
+        if (enqueue_step(h, st, d, mp, mi, false, small)) return KDT_ERR_CUDA;
         if (timed) CK(cudaEventRecord(h->ev3, st));
     }
-    h->stats.kernel_launches += 4 + ((h->cfg.plan & PLAN_ORDER) ? 2 : 0) +
+    h->stats.kernel_launches += small ? 3 : 4 + ((h->cfg.plan & PLAN_ORDER) ? 2 : 0) +
                                 ((h->cfg.plan & PLAN_ORDER) || (h->prop_on && (h->cfg.plan & PLAN_NETWORK)) ? 1 : 0) +
                                 (h->prop_on && (h->cfg.plan & PLAN_NETWORK) && (h->cfg.plan & PLAN_TENSOR) ? 1 : 0) +
-                                (h->qhist ? h->qD + 5 : 0) + (step_in_rounds(h) ? 2 * h->rm_rounds + 1 : 0);
+                                (h->qhist ? h->qD + 5 : 0) + (rounds ? 2 * h->rm_rounds + 1 : 0);
     CK(cudaStreamSynchronize(st));
     if (h->qhist) h->ncells = h->qleaves = h->hscal[S_NCELLS];
     if (timed) {
@@ -1482,7 +1553,7 @@ int build_quadtree(kdt *h)
     int init_bbox[4] = {INT_MAX, INT_MAX, INT_MIN, INT_MIN};
     CK(cudaMemsetAsync(h->scal, 0, S_NUM * sizeof(int), st));
     CK(cudaMemcpyAsync(h->scal + S_MINX, init_bbox, sizeof init_bbox, cudaMemcpyHostToDevice, st));
-    k_range<<<thread_grid(h, n, 256), 256, 0, st>>>(h->xy, n, h->cfg.domain_bits, h->scal + S_STATUS,
+    k_range<<<std::min(thread_grid(h, n, 256), 4 * sm_count(h->device)), 256, 0, st>>>(h->xy, n, h->cfg.domain_bits, h->scal + S_STATUS,
                                                     h->scal + S_MINX);
     if (sync_scalars(h)) return KDT_ERR_CUDA;
     const int x0 = h->hscal[S_MINX], y0 = h->hscal[S_MINY];
@@ -1565,7 +1636,10 @@ int build_impl(kdt *h, const int32_t *xy, const int64_t *offs, int n_inst)
 {
     CK(cudaSetDevice(h->device));
     if (foreign(h, xy)) return KDT_ERR_ARG;
-    free_state(h);
+    // the last build's arrays when they have the room and are not four times too large
+    // (allocating and freeing them took 2 of the 12 ms of a build of 1e6 points)
+    if (h->n_room >= offs[n_inst] && h->n_room / 4 <= offs[n_inst] && h->inst_room >= n_inst) reset_state(h);
+    else free_state(h);
     int rc = alloc_state(h, offs, n_inst);
     if (rc) {
         free_state(h);

@@ -51,7 +51,9 @@ struct Inst {
                       // index order
     int ninst;
     const int *pending;  // a step whose moves went through rounds: how many of them are left to
-                         // the kinetic kernel (in the partitions' lists); null: all of them
+                         // the kinetic kernel; null: all of them
+    const int *left;     // ... few of them (at most few_left): a list, ticket k takes move left[k];
+    int few_left;        // more: the partitions' lists
 };
 
 // Partition of a position of instance `inst`: its grid cell, or the quad-tree leaf of
@@ -288,16 +290,22 @@ __device__ __forceinline__ const int3 *step_moves(const Dev &d, const int3 *move
 
 // Start of a step: the scalars and the rounds' counters zero, every partition's move list
 // empty, every deferred entry -1 (one launch instead of several memsets).
-__global__ void k_step_clear(int *scal, int nscal, int *head, int ncells, int4 *deferred, int ndef, int *rounds,
-                             int nrounds)
+__device__ __forceinline__ void step_clear(int *scal, int nscal, int *head, int ncells, int4 *deferred, int ndef,
+                                           int *rounds, int nrounds, int tid, int nthreads)
 {
-    const int stride = gridDim.x * blockDim.x;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < max(max(ncells, ndef), nrounds); i += stride) {
+    for (int i = tid; i < max(max(ncells, ndef), max(nscal, nrounds)); i += nthreads) {
         if (i < nscal) scal[i] = 0;
         if (i < nrounds) rounds[i] = 0;
         if (i < ncells) head[i] = -1;
         if (i < ndef) deferred[i] = make_int4(-1, -1, -1, -1);
     }
+}
+
+__global__ void k_step_clear(int *scal, int nscal, int *head, int ncells, int4 *deferred, int ndef, int *rounds,
+                             int nrounds)
+{
+    step_clear(scal, nscal, head, ncells, deferred, ndef, rounds, nrounds, blockIdx.x * blockDim.x + threadIdx.x,
+               gridDim.x * blockDim.x);
 }
 
 // An invalid move stops the step; it wins over the displacement rule's DEV_FAR, so
@@ -316,16 +324,12 @@ __device__ __forceinline__ void intake_fail(int *status, int code)
 // is counted, and the
 // step becomes a rebuild (DEV_FAR stops the kinetic kernel before it changes anything).
 // head null: no lists (the moves go through rounds first, which link what they leave).
-__global__ void k_intake_link(Dev d, const int3 *moves, int m, Inst I, int bits, int *head, int *next,
-                              int2 *old_xy, int3 *gmoves, const unsigned long long *dloc2, double far2)
+__device__ __forceinline__ void intake(const Dev &d, const int3 *moves, int m, const Inst &I, int bits, int *head,
+                                       int *next, int2 *old_xy, int3 *gmoves, const unsigned long long *dloc2,
+                                       double far2, int tid, int nthreads)
 {
-    if (d.ctl) {
-        m = __ldcg(d.ctl);
-        d.stamp = __ldcg(d.ctl + 1);
-    }
-    moves = step_moves(d, moves);
     long long lim = 1ll << bits;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
+    for (int i = tid; i < m; i += nthreads) {
         int inst = I.ninst > 1 ? csr_find(I.moff, I.ninst + 1, i) : 0;
         int p0 = I.pofs[inst], ni = I.pofs[inst + 1] - p0;
         int3 mv = moves[i];
@@ -362,6 +366,17 @@ __global__ void k_intake_link(Dev d, const int3 *moves, int m, Inst I, int bits,
         }
         if (head) next[i] = atomicExch(head + cell, i);
     }
+}
+
+__global__ void k_intake_link(Dev d, const int3 *moves, int m, Inst I, int bits, int *head, int *next,
+                              int2 *old_xy, int3 *gmoves, const unsigned long long *dloc2, double far2)
+{
+    if (d.ctl) {
+        m = __ldcg(d.ctl);
+        d.stamp = __ldcg(d.ctl + 1);
+    }
+    intake(d, step_moves(d, moves), m, I, bits, head, next, old_xy, gmoves, dloc2, far2,
+           blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 // ------------------------------------------------------------------ step: kinetic
@@ -612,7 +627,9 @@ __global__ void __launch_bounds__(WPB * 32, MINB) k_kinetic(Dev dp, const int3 *
                                                             int4 *deferred, int *defer_count, int defer_cap,
                                                             int *viol, int viol_cap)
 {
-    if (I.pending && __ldcg(I.pending) == 0) return;  // the rounds did every move
+    const int npend = I.pending ? __ldcg(I.pending) : 0;
+    if (I.pending && npend == 0) return;  // the rounds did every move
+    const bool few = I.pending && npend <= I.few_left;
     KD_BLOCK_DEV(dp);
     __shared__ WarpShared shs[WPB];
     int wib = threadIdx.x >> 5;
@@ -621,7 +638,7 @@ __global__ void __launch_bounds__(WPB * 32, MINB) k_kinetic(Dev dp, const int3 *
     Warp w = make_warp(&shs[wib], gw + 1, gw + 17 * d.stamp, d);
     const bool tl = d.timeline && d.counters;
     if (tl && gw == 0 && w.lane == 0) d.counters[C_T0] = global_ns();
-    const int items = (I.ncells_dyn ? __ldcg(I.ncells_dyn) : ncells) * wpp;
+    const int items = few ? npend : (I.ncells_dyn ? __ldcg(I.ncells_dyn) : ncells) * wpp;
     // One loop, one move per iteration: first the moves of the (partition, share) work
     // items the warp takes from a ticket; when those are gone, the whole moves left
     // so far (drained in parallel with the warps still busy; each may be left again,
@@ -634,7 +651,7 @@ __global__ void __launch_bounds__(WPB * 32, MINB) k_kinetic(Dev dp, const int3 *
         int2 q;
         if (tickets) {
             // next move of this work item (every wpp-th of the partition's list)
-            if (i >= 0) i = __shfl_sync(FULL, __ldcg(next + i), 0);
+            if (i >= 0) i = few ? -1 : __shfl_sync(FULL, __ldcg(next + i), 0);
             while (i >= 0 && ++kk % wpp != sub) i = __shfl_sync(FULL, __ldcg(next + i), 0);
             if (i < 0) {
                 if (read_status(d)) break;
@@ -648,16 +665,22 @@ __global__ void __launch_bounds__(WPB * 32, MINB) k_kinetic(Dev dp, const int3 *
                     if (__shfl_sync(FULL, w.lane == 0 ? __ldcg(defer_count) : 0, 0) == 0) break;
                     continue;
                 }
-                c = t / wpp;
-                sub = t - c * wpp;
-                if (I.order) c = __ldcg(I.order + c);
-                else if (I.stride > 1) c = (int)(((long long)c * I.stride) % ncells);
-                kk = -1;
-                i = __shfl_sync(FULL, __ldcg(head + c), 0);
-                int inst = I.ninst > 1 ? csr_find(I.cofs, I.ninst + 1, c) : 0;
-                set_instance(w, I.pofs[inst], I.pofs[inst + 1] - I.pofs[inst]);
-                while (i >= 0 && ++kk % wpp != sub) i = __shfl_sync(FULL, __ldcg(next + i), 0);
-                if (i < 0) continue;
+                if (few) {
+                    i = __shfl_sync(FULL, __ldcg(I.left + t), 0);
+                    const int inst = I.ninst > 1 ? csr_find(I.pofs, I.ninst + 1, moves[i].x) : 0;
+                    set_instance(w, I.pofs[inst], I.pofs[inst + 1] - I.pofs[inst]);
+                } else {
+                    c = t / wpp;
+                    sub = t - c * wpp;
+                    if (I.order) c = __ldcg(I.order + c);
+                    else if (I.stride > 1) c = (int)(((long long)c * I.stride) % ncells);
+                    kk = -1;
+                    i = __shfl_sync(FULL, __ldcg(head + c), 0);
+                    int inst = I.ninst > 1 ? csr_find(I.cofs, I.ninst + 1, c) : 0;
+                    set_instance(w, I.pofs[inst], I.pofs[inst + 1] - I.pofs[inst]);
+                    while (i >= 0 && ++kk % wpp != sub) i = __shfl_sync(FULL, __ldcg(next + i), 0);
+                    if (i < 0) continue;
+                }
             }
             int3 mv = moves[i];
             p = mv.x;
@@ -919,6 +942,7 @@ __global__ void k_range(const int2 *xy, int n, int bits, int *status, int *bbox)
         mxx = max(mxx, __shfl_xor_sync(FULL, mxx, o));
         mxy = max(mxy, __shfl_xor_sync(FULL, mxy, o));
     }
+    // (a few blocks a SM: an atomic per warp and side of 1e6 points queued for 70 us)
     if ((threadIdx.x & 31) == 0) {
         atomicMin(bbox + 0, mnx);
         atomicMin(bbox + 1, mny);
@@ -974,7 +998,7 @@ __global__ void k_place_order(int n, const unsigned *key, const int *off, int *f
 __global__ void k_third(const int2 *xy, int n, const int *order, int *third)
 {
     int2 a = xy[order[0]], b = xy[order[1]];
-    for (int j = 2 + blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
+    for (int j = 2 + blockIdx.x * blockDim.x + threadIdx.x; j < n && j < __ldcg(third); j += gridDim.x * blockDim.x)
         if (orient2d(a, b, xy[order[j]]) != 0) atomicMin(third, j);
 }
 
@@ -1010,18 +1034,47 @@ __global__ void k_init(Dev d, const int *order, const int *third, int *tri_count
 // inside its own range of `order`), per-instance first triangles, and rounds of insertions
 // over all instances (kdt_rounds.cuh), level by level.
 
-// bounding box of every instance (bbox[4 i .. 4 i + 3]) and the range check
+// bounding box of every instance (bbox[4 i .. 4 i + 3]) and the range check: a warp takes a
+// run of RANGE_RUN points and, while they are of one instance, keeps its box in registers
+constexpr int RANGE_RUN = 1024;
+
+__device__ __forceinline__ void range_flush(int *b, int mnx, int mny, int mxx, int mxy)
+{
+    mnx = __reduce_min_sync(FULL, mnx);
+    mny = __reduce_min_sync(FULL, mny);
+    mxx = __reduce_max_sync(FULL, mxx);
+    mxy = __reduce_max_sync(FULL, mxy);
+    if ((threadIdx.x & 31) == 0 && mnx <= mxx) {
+        atomicMin(b + 0, mnx);
+        atomicMin(b + 1, mny);
+        atomicMax(b + 2, mxx);
+        atomicMax(b + 3, mxy);
+    }
+}
+
 __global__ void k_range_batch(const int2 *xy, int n, const int *pofs, int ninst, int bits, int *status, int *bbox)
 {
     const long long lim = 1ll << bits;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int2 p = xy[i];
-        if (p.x < 0 || p.y < 0 || p.x >= lim || p.y >= lim) atomicCAS(status, 0, DEV_RANGE);
-        int *b = bbox + 4 * csr_find(pofs, ninst + 1, i);
-        atomicMin(b + 0, p.x);
-        atomicMin(b + 1, p.y);
-        atomicMax(b + 2, p.x);
-        atomicMax(b + 3, p.y);
+    const int lane = threadIdx.x & 31, warps = gridDim.x * (blockDim.x >> 5);
+    for (int run = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); (long long)run * RANGE_RUN < n; run += warps) {
+        const int lo = run * RANGE_RUN, hi = min(n, lo + RANGE_RUN);
+        int inst = csr_find(pofs, ninst + 1, lo);
+        for (int i0 = lo; i0 < hi;) {
+            // the part of the run that is this instance's
+            const int end = min(hi, __ldg(pofs + inst + 1));
+            int mnx = INT_MAX, mny = INT_MAX, mxx = INT_MIN, mxy = INT_MIN;
+            for (int i = i0 + lane; i < end; i += 32) {
+                const int2 p = xy[i];
+                if (p.x < 0 || p.y < 0 || p.x >= lim || p.y >= lim) atomicCAS(status, 0, DEV_RANGE);
+                mnx = min(mnx, p.x);
+                mny = min(mny, p.y);
+                mxx = max(mxx, p.x);
+                mxy = max(mxy, p.y);
+            }
+            range_flush(bbox + 4 * inst, mnx, mny, mxx, mxy);
+            i0 = end;
+            ++inst;
+        }
     }
 }
 
@@ -1052,7 +1105,7 @@ __global__ void k_third_batch(const int2 *xy, int n, const int *order, const int
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         const int inst = csr_find(pofs, ninst + 1, j);
         const int p0 = pofs[inst];
-        if (j - p0 < 2) continue;
+        if (j - p0 < 2 || j - p0 >= __ldcg(third + inst)) continue;
         if (orient2d(xy[order[p0]], xy[order[p0 + 1]], xy[order[j]]) != 0) atomicMin(third + inst, j - p0);
     }
 }
@@ -1147,7 +1200,7 @@ __global__ void k_exp_sortseg(int n, const int *off, const int *cnt, int3 *out)
 // sorted by one block in shared memory and written in one piece.
 // GB300, list of 16e6 points into device memory: 3.29 ms placed (count 0.30, place 1.32, sort
 // 1.45), 1.67 ms in buckets; 512 instances, 21.7e6 points: 3.24 -> 2.04; 1e6 points: 215 ->
-// 175 us; 1,000 points: 80 -> 48 us (four launches and one wait instead of eight and two).
+// 155 us; 1,000 points: 80 -> 46 us (four launches and one wait instead of eight and two).
 constexpr int EXB_ROWS = 7;     // rows a bucket may hold per first id (mean 2, up to 6 at the lowest ids)
 constexpr int EXB_SHIFT = 9;    // largest s: 33 KB a block
 constexpr int EXB_THREADS = 256;

@@ -145,21 +145,17 @@ __device__ __forceinline__ int near_start(const Dev &d, const int *order, int n,
 // itself, so no warp is as long as the union of two operations' paths.  An operation
 // outside RL's limits is planned again, by the 32-lane form when LAST is set or later, and
 // with LAST goes to the list of the warp-wide path.
+//
+// round_plan: `tid` of `nthreads` threads (whole warps), shared: one RegionShared per group of
+// the block.
 template <int MODE, int RL>
-__global__ void __launch_bounds__(ROUND_THREADS, ROUND_BLOCKS) k_round_plan(Dev d, Rounds R, int b, RoundMoves M, RoundBuild B,
-                                                              int last)
+__device__ __forceinline__ void round_plan(const Dev &d, const Rounds &R, int b, const RoundMoves &M,
+                                           const RoundBuild &B, int total, int last, RegionShared<RL> *shared, int tid,
+                                           int nthreads)
 {
     constexpr bool MOVE = MODE != REGION_INSERT;
-    if (__ldcg(d.status)) return;
-    __shared__ RegionShared<RL> shared[ROUND_THREADS / RL];
-    int total = B.total;
-    if (MOVE && d.ctl) {
-        total = __ldcg(d.ctl);
-        d.stamp = __ldcg(d.ctl + 1);
-    }
     int nlost, head, count;
     round_window(R, b, total, nlost, head, count);
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int off = __ldcg(R.off + b);
     if (tid == 0) {
         R.head[b + 1] = head + count - nlost;
@@ -168,7 +164,7 @@ __global__ void __launch_bounds__(ROUND_THREADS, ROUND_BLOCKS) k_round_plan(Dev 
     constexpr int PER_WARP = 32 / RL;
     const int l = threadIdx.x & (RL - 1), g0 = threadIdx.x & 31 & ~(RL - 1);
     const unsigned gm = (FULL >> (32 - RL)) << g0;
-    const int warps = gridDim.x * (ROUND_THREADS / 32);
+    const int warps = nthreads / 32;
     const bool alone = count <= warps;
     if (alone && g0) return;
     RegionShared<RL> &sh = shared[threadIdx.x / RL];
@@ -233,22 +229,36 @@ __global__ void __launch_bounds__(ROUND_THREADS, ROUND_BLOCKS) k_round_plan(Dev 
     if (steps) atomicAdd(d.counters + C_WALK_STEPS, (unsigned long long)steps);
 }
 
+template <int MODE, int RL>
+__global__ void __launch_bounds__(ROUND_THREADS, ROUND_BLOCKS) k_round_plan(Dev d, Rounds R, int b, RoundMoves M,
+                                                                            RoundBuild B, int last)
+{
+    if (__ldcg(d.status)) return;
+    __shared__ RegionShared<RL> shared[ROUND_THREADS / RL];
+    int total = B.total;
+    if (MODE != REGION_INSERT && d.ctl) {
+        total = __ldcg(d.ctl);
+        d.stamp = __ldcg(d.ctl + 1);
+    }
+    round_plan<MODE, RL>(d, R, b, M, B, total, last, shared, blockIdx.x * blockDim.x + threadIdx.x,
+                         gridDim.x * ROUND_THREADS);
+}
+
 // ROUND_LANES lanes per operation, lane l its triangles l, l + 8, ...  The owner
 // words keep the priorities (a neighbour that checks its own border meanwhile must still
 // see them).
 template <bool MOVE>
-__global__ void __launch_bounds__(256) k_round_commit(Dev d, Rounds R, int b, RoundMoves M, RoundBuild B)
+__device__ __forceinline__ void round_commit(const Dev &d, const Rounds &R, int b, const RoundMoves &M, int total,
+                                             int *sum, int tid, int nthreads)
 {
-    if (__ldcg(d.status)) return;
-    const int total = MOVE && d.ctl ? __ldcg(d.ctl) : B.total;
     int nlost, head, count;
     round_window(R, b, total, nlost, head, count);
     const int lane = threadIdx.x & (ROUND_LANES - 1);
     const unsigned gm = 0xffu << (threadIdx.x & 24);  // this operation's lanes
     int nwin = 0, nlose = 0, degs = 0, flips = 0, edges = 0, ghosts = 0, props = 0, hits = 0;
-    const int groups = gridDim.x * (blockDim.x / ROUND_LANES);
+    const int groups = nthreads / ROUND_LANES;
     // (whole warps take part in the ballots: the loop ends for a warp at once)
-    for (int x0 = (blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / ROUND_LANES; x0 < count; x0 += groups) {
+    for (int x0 = (tid & ~31) / ROUND_LANES; x0 < count; x0 += groups) {
         const int x = x0 + ((threadIdx.x & 31) / ROUND_LANES);
         int4 h = make_int4(-1, -1, 0, 0);
         if (x < count) h = __ldcg(R.hdr + x);
@@ -305,7 +315,6 @@ __global__ void __launch_bounds__(256) k_round_commit(Dev d, Rounds R, int b, Ro
         }
     }
     if (!d.counters) return;
-    __shared__ int sum[8];
     if (threadIdx.x < 8) sum[threadIdx.x] = 0;
     __syncthreads();
     const int part[8] = {nwin, nlose, degs, flips, edges, ghosts, props, hits};
@@ -324,16 +333,25 @@ __global__ void __launch_bounds__(256) k_round_commit(Dev d, Rounds R, int b, Ro
     }
 }
 
-// After the last of `rounds` rounds of a step: the owner words of every operation's
-// slots zero, and the moves not done (left out, losers of the last round, fresh items never
-// taken) onto the lists of their partitions, for the kinetic kernel: a partition's moves
-// run one after another there, so moves that meet do not compete.
-__global__ void k_round_clear(Dev d, Rounds R, int rounds, int m, Inst I, int bits, const int3 *gmoves,
-                              const int2 *old_xy, int *head, int *next)
+template <bool MOVE>
+__global__ void __launch_bounds__(256) k_round_commit(Dev d, Rounds R, int b, RoundMoves M, RoundBuild B)
 {
     if (__ldcg(d.status)) return;
-    if (d.ctl) m = __ldcg(d.ctl);
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthreads = gridDim.x * blockDim.x;
+    __shared__ int sum[8];
+    round_commit<MOVE>(d, R, b, M, MOVE && d.ctl ? __ldcg(d.ctl) : B.total, sum, blockIdx.x * blockDim.x + threadIdx.x,
+                       gridDim.x * blockDim.x);
+}
+
+// After the last of `rounds` rounds of a step: the owner words of every operation's
+// slots zero, and the moves not done (left out, losers of the last round, fresh items never
+// taken) to the kinetic kernel: few of them as a list, more on the lists of their
+// partitions, whose moves run one after another, so that moves that meet do not compete
+// (all 3,000 points of one partition moving at once filled the list of moves left for
+// later when every warp took one; 85,000 partitions' empty lists cost 100 us to look at).
+__device__ __forceinline__ void round_clear(const Dev &d, const Rounds &R, int rounds, int m, const Inst &I, int bits,
+                                            const int3 *gmoves, const int2 *old_xy, int *head, int *next, int tid,
+                                            int nthreads)
+{
     const long long words = (long long)__ldcg(R.off + rounds) * RT;
     for (long long i = 4ll * tid; i < words; i += 4ll * nthreads) {
         const int4 s = __ldcg(reinterpret_cast<const int4 *>(R.slots + i));
@@ -349,8 +367,66 @@ __global__ void k_round_clear(Dev d, Rounds R, int rounds, int m, Inst I, int bi
         const int item = i < nleft ? __ldcg(R.left + i)
                                    : (i < nleft + nlost ? __ldcg(R.lost[rounds & 1] + i - nleft) : fresh + i - nleft - nlost);
         const int inst = I.ninst > 1 ? csr_find(I.pofs, I.ninst + 1, gmoves[item].x) : 0;
-        next[item] = atomicExch(head + partition_of(I, inst, bits, old_xy[item]), item);
+        if (pending <= I.few_left) R.left[i] = item;
+        else next[item] = atomicExch(head + partition_of(I, inst, bits, old_xy[item]), item);
     }
+}
+
+__global__ void k_round_clear(Dev d, Rounds R, int rounds, int m, Inst I, int bits, const int3 *gmoves,
+                              const int2 *old_xy, int *head, int *next)
+{
+    if (__ldcg(d.status)) return;
+    round_clear(d, R, rounds, d.ctl ? __ldcg(d.ctl) : m, I, bits, gmoves, old_xy, head, next,
+                blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+// A whole small step in one block: clearing, intake, rounds until every move is done (or a
+// round does none), and what is left to the kinetic kernel.  The kernels it replaces take
+// 2 to 4 us each whatever they do, and a step of a few moves is three rounds of them: 1,000
+// points, 13 moves, 67 -> 61 us a step with a wait after each, 500 -> 450 us for eight and an
+// export.
+constexpr int SMALL_MOVES = 64;      // two moves a warp, one after the other
+constexpr int SMALL_THREADS = 512;
+constexpr int SMALL_ROUNDS = 16;
+constexpr int SMALL_CELLS = 8192;    // partitions one block clears in passing
+
+__global__ void __launch_bounds__(SMALL_THREADS) k_step_small(Dev d, const int3 *moves, int m, Inst I, int bits,
+                                                              int *scal, int nscal, int *head, int ncells, int *next,
+                                                              int4 *deferred, int ndef, int2 *old_xy, int3 *gmoves,
+                                                              const unsigned long long *dloc2, double far2, Rounds R,
+                                                              int *counters, int ncounters)
+{
+    __shared__ RegionShared<32> shared[SMALL_THREADS / 32];
+    __shared__ int sum[8];
+    const int tid = threadIdx.x;
+    if (d.ctl) {
+        m = __ldcg(d.ctl);
+        d.stamp = __ldcg(d.ctl + 1);
+    }
+    // (every phase's writes are seen by the next one's: one block, a fence, a barrier)
+    auto phase = [] {
+        __threadfence();
+        __syncthreads();
+    };
+    step_clear(scal, nscal, head, ncells, deferred, ndef, counters, ncounters, tid, SMALL_THREADS);
+    phase();
+    intake(d, step_moves(d, moves), m, I, bits, nullptr, next, old_xy, gmoves, dloc2, far2, tid, SMALL_THREADS);
+    phase();
+    if (__ldcg(d.status)) return;
+    const RoundMoves M{gmoves};
+    const RoundBuild B{};
+    int b = 0;
+    for (int pending = m; b < SMALL_ROUNDS;) {
+        round_plan<REGION_MOVE, 32>(d, R, b, M, B, m, 1, shared, tid, SMALL_THREADS);
+        phase();
+        round_commit<true>(d, R, b, M, m, sum, tid, SMALL_THREADS);
+        phase();
+        ++b;
+        const int now = __ldcg(R.lostcnt + b) + m - __ldcg(R.head + b);
+        if (now == 0 || now == pending) break;
+        pending = now;
+    }
+    round_clear(d, R, b, m, I, bits, gmoves, old_xy, head, next, tid, SMALL_THREADS);
 }
 
 // the owner words of slots [s0, s0 + n) zero (after the rounds of a build)
