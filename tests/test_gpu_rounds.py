@@ -147,3 +147,85 @@ def test_export_buckets(n, hub):
         with pytest.raises(kdt.KDTError) as e:
             t.export_triangles(out[:got.shape[0] - 1])
         assert e.value.name == "KDT_ERR_CAPACITY" and int((out != -1).sum()) == 0
+
+
+@pytest.mark.parametrize("grid", [90, 91])
+@pytest.mark.parametrize("m", [1, 2, 63, 64, 65])
+def test_small_step_limits(grid, m):
+    """One block's steps (up to 64 moves, up to 8192 partitions) and those just past them."""
+    w = W.KineticWorkload(W.uniform_points(700, 18, m), grid, 18, (0, 0), (1, 1), seed=3)
+    xy = np.array(w.positions)
+    rng = np.random.default_rng(m)
+    t = _tri(grid=grid, domain_bits=18, rebuild_ratio=2.0)
+    t.build(xy)
+    for s in range(4):
+        ids = rng.choice(len(xy), size=m, replace=False)
+        new = xy.copy()
+        new[ids] = (new[ids] + rng.integers(-9000, 9001, size=(m, 2))).clip(0, (1 << 18) - 1)
+        both = np.concatenate([xy, new[ids]])
+        assert np.unique(both, axis=0).shape[0] == len(both)
+        xy = new.astype(np.int32)
+        t.step(np.concatenate([ids[:, None], xy[ids]], 1).astype(np.int32))
+        assert_same(t.export_triangles(), xy, "grid %d m %d step %d" % (grid, m, s))
+    st = t.stats()
+    assert t.verify() == 0 and st["fallbacks"] == 0 and st["rebuilds"] == 1
+
+
+@pytest.mark.parametrize("hubs", [255, 256, 257])
+def test_leftovers_as_list_or_by_partition(hubs):
+    """Hubs of degree 40 (more triangles than a round's lanes hold) all go to the kinetic
+    kernel: as a list up to a quarter of the least room for moves (256), else by partition."""
+    i = np.arange(17 * 17)[:hubs]
+    c = np.stack([70000 + 100000 * (i % 17), 70000 + 100000 * (i // 17)], 1)
+    a = 2 * np.pi * (np.arange(40) + 0.3) / 40
+    r = 20000.0 + 7 * (np.arange(40) % 5)
+    rim = np.rint(np.stack([r * np.cos(a), r * np.sin(a)], 1)).astype(np.int64)
+    xy = np.concatenate([c, (c[:, None] + rim[None]).reshape(-1, 2)]).astype(np.int32)
+    tri = oracle.delaunay(xy)
+    assert (np.bincount(tri.ravel(), minlength=len(xy))[:hubs] >= 40).all()
+    t = _tri(grid=4, domain_bits=21, rebuild_ratio=2.0)
+    t.build(xy)
+    for s in range(3):
+        xy[:hubs] += np.array([3, -2], np.int32)
+        t.step(np.concatenate([i[:, None], xy[:hubs]], 1).astype(np.int32))
+        assert_same(t.export_triangles(), xy, "%d hubs step %d" % (hubs, s))
+    assert t.verify() == 0 and t.stats()["fallbacks"] == 0
+
+
+@pytest.mark.parametrize("quadtree", [0, 1, 2])
+def test_arrays_kept_between_builds(quadtree):
+    """One handle over point sets that fit the last one's arrays, that do not, that are far
+    smaller, batches of them, and one that is refused: a step after each, exact."""
+    from paper_2308_06484_gb300 import kdt
+    t = _tri(domain_bits=20, points_per_partition=64, quadtree=quadtree, rebuild_ratio=2.0)
+    rng = np.random.default_rng(1)
+
+    def moved(xy):
+        new = xy.copy()
+        ids = rng.choice(len(xy), size=max(1, len(xy) // 20), replace=False)
+        new[ids] = (new[ids] + rng.integers(-3000, 3001, size=(ids.size, 2))).clip(0, (1 << 20) - 1)
+        assert np.unique(np.concatenate([xy, new[ids]]), axis=0).shape[0] == len(xy) + ids.size
+        return new.astype(np.int32), np.concatenate([ids[:, None], new[ids]], 1).astype(np.int32)
+
+    for k, sizes in enumerate([(5000,), (4000,), (1300,), (1000,), (20000,), (300, 800, 3), (900,), None, (700,),
+                               (3,), (40, 50), (6000,)]):
+        if sizes is None:
+            dup = W.uniform_points(800, 20, 9)
+            dup[5] = dup[700]
+            with pytest.raises(kdt.KDTError) as e:
+                t.build(dup)
+            assert e.value.name == "KDT_ERR_DUPLICATE"
+            continue
+        xys = [W.uniform_points(n, 20, 10 * k + j) for j, n in enumerate(sizes)]
+        if len(xys) == 1:
+            t.build(xys[0])
+            new, mv = moved(xys[0])
+            t.step(mv)
+            assert_same(t.export_triangles(), new, "build %d" % k)
+        else:
+            t.build_batch(xys)
+            parts = [moved(x) for x in xys]
+            t.step_batch(np.concatenate([p[1] for p in parts]), np.cumsum([0] + [len(p[1]) for p in parts]))
+            for j, p in enumerate(parts):
+                assert_same(t.export_triangles_inst(j), p[0], "build %d instance %d" % (k, j))
+        assert t.verify() == 0
