@@ -222,6 +222,11 @@ def test_arrays_kept_between_builds(quadtree):
             new, mv = moved(xys[0])
             t.step(mv)
             assert_same(t.export_triangles(), new, "build %d" % k)
+        elif quadtree:  # (one point set only: refused, the triangulation stays as it was)
+            with pytest.raises(kdt.KDTError) as e:
+                t.build_batch(xys)
+            assert e.value.name == "KDT_ERR_ARG"
+            assert_same(t.export_triangles(), new, "build %d" % k)
         else:
             t.build_batch(xys)
             parts = [moved(x) for x in xys]
