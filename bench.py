@@ -343,7 +343,7 @@ def timed_steps(tri, moves, warmup, flush=None, stepper=None):
 
 def kernel_pass(make_tri, xy0, moves, warmup, flush=None, stepper=None):
     """The same steps on an instrumented handle (timing = 1): mean event-timed duration
-    of the kinetic kernel, and the handle's counters."""
+    of a step's rounds and kinetic kernel, and the handle's counters."""
     tri = make_tri(timing=1)
     tri.build(xy0)
     timed_steps(tri, moves, warmup, flush, stepper=(lambda m: stepper(tri, m)) if stepper else None)
@@ -356,7 +356,8 @@ def roofline(bpu, moves_per_launch, kernel_ms, traffic):
     peak, kind = measured_peaks()
     achieved = bpu * moves_per_launch / (kernel_ms / 1000.0) / 1e9
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-            "traffic": traffic, "kernel": "k_kinetic", "kernel_ms": kernel_ms, "bytes_per_update": bpu,
+            "traffic": traffic, "kernel": "rounds (k_round_plan, k_round_commit, k_round_clear) + k_kinetic",
+            "kernel_ms": kernel_ms, "bytes_per_update": bpu,
             "moves_per_launch": moves_per_launch, "peak_kind": kind + " (hbm_gbs, copy bandwidth)"}
 
 

@@ -78,7 +78,8 @@ typedef struct {
     float rebuild_ratio;   /* m / n above which a step is done as a full rebuild (0.25)     */
     int32_t filter;        /* 1: FP32 filter in front of the exact incircle (default)       */
     int32_t verify;        /* 1: run the full GPU verifier after every step (tests)         */
-    int32_t timing;        /* 1: time the kinetic kernel with CUDA events (kdt_stats)       */
+    int32_t timing;        /* 1: time the rounds of moves and the kinetic kernel with CUDA
+                              events (kdt_stats)                                            */
     int32_t warps_per_block; /* kinetic kernel launch shape (default 4)                      */
     int32_t build_warps;   /* warps inserting concurrently during a build (0 = auto)         */
     int32_t kinetic_warps; /* warps moving points concurrently in a step (0 = one per cell)  */
@@ -149,7 +150,8 @@ typedef struct {
     int32_t batch_build;   /* 1 (default): the instances of a batch are (re)built together,
                               one set of launches for all of them; 0: one instance after
                               another.  The triangulations are the same.                    */
-    int32_t kinetic_blocks_per_sm; /* 0 or 6 (default): the kinetic kernel compiled for six
+    int32_t kinetic_blocks_per_sm; /* 0 or 6 (default): the kinetic kernel (the moves that the
+                              rounds of kdt_rounds.cuh leave, or all) compiled for six
                               128-thread blocks per SM (up to 80 registers a thread); 7: for
                               seven (up to 72 registers, more warps in flight).  Scheduling
                               only.                                                          */
@@ -167,7 +169,8 @@ typedef struct {
     int64_t flips, retries, walk_steps, exact_incircle, sos_ties, deferred;
     int64_t violations, fixup_flips, deleted_degree_sum, stack_drops, edge_splits;
     int64_t ghost_splits, deletes, inserts, flip_tests;
-    double kinetic_kernel_ms; /* sum of event-timed kinetic kernel durations (timing = 1) */
+    double kinetic_kernel_ms; /* sum of event-timed durations of a step's rounds and kinetic
+                                 kernel (timing = 1)                                      */
     int64_t kinetic_kernel_timed; /* launches included in kinetic_kernel_ms               */
     int64_t last_fallback_reason; /* internal status that triggered the last fallback     */
     int64_t last_fallback_point;  /* point whose operation reported it (-1 if unknown)     */

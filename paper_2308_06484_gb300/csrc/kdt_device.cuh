@@ -13,7 +13,8 @@
 //   xy[p] = int2 position, pt_tri[p] = an incident live triangle (-1 while p is
 //   deleted inside a step).
 //
-// Execution model.  One warp runs one operation.  Control flow is warp-uniform:
+// Execution model (of this file's operations, which do what the rounds of kdt_rounds.cuh
+// leave: large stars, the hull, the variants).  One warp runs one operation.  Control flow is warp-uniform:
 // every lane computes the same sequential logic on the same values, global reads
 // are done by one or several lanes and broadcast with shuffles, global writes are
 // issued by lane 0, and lane-parallel sections (claims, loads, ear tests) combine

@@ -1,10 +1,13 @@
 // Kernels of the kinetic Delaunay library.  Included once, by kdt.cu.
 //
-//   step:    k_intake_link -> k_kinetic (last warp: deferred points, certification of
-//            global-path writes) (-> k_fixup / k_certify until no violation)
+//   step:    k_step_clear -> k_intake_link -> rounds of moves (kdt_rounds.cuh) -> k_kinetic
+//            for what they leave, or for every move of the forms they do not take (last warp:
+//            deferred points, certification of global-path writes) (-> k_fixup / k_certify
+//            until no violation); a step of a few moves: k_step_small -> k_kinetic
 //   build:   k_range / k_bbox -> k_hilbert -> scan -> k_place_order -> k_third -> k_init
 //            -> rounds of insertions (kdt_rounds.cuh) -> k_certify_all (-> k_fixup ...)
-//   export:  k_exp_count -> scan -> k_exp_place -> k_exp_sortseg
+//   export:  k_exb_* (buckets of first ids); without allocations, and where a bucket is too
+//            large for a block: k_exp_count -> scan -> k_exp_place -> k_exp_sortseg
 #pragma once
 #include "kdt_local.cuh"
 

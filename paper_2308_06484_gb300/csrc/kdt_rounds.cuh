@@ -31,7 +31,7 @@
 //   step, 512 instances, 212,000 moves            2.6 -> 0.8 ms
 //   step, 2e5 points, 1,950 moves that leave their star   390 -> 180 us
 //   rebuild, 1e6 uniform points                  28.8 -> 10.5 ms
-//   rebuild, 128 instances, 1.5e6 points         37   -> 11.9 ms
+//   rebuild, 128 instances, 1.5e6 points         37   -> 9.8 ms
 // Bound now: the latency of the plan's chain (12-27 us a round of a few thousand operations)
 // times the number of rounds; with 1e5 operations or more, the SMs' issue slots (41 %
 // busy) and the spread of the loads over L2.
