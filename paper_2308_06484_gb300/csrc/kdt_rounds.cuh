@@ -458,23 +458,33 @@ __global__ void k_build_rest(Rounds R, int b, RoundBuild B)
         R.left[atomicAdd(R.left_count, 1)] = i < nlost ? __ldcg(R.lost[b & 1] + i) : __ldg(B.queue + head + i - nlost);
 }
 
-// Points the rounds left out (a cavity above their limits), one warp per insertion: the
-// staged Bowyer-Watson insertion, else split and flips, with claims by compare-and-swap.
-// Each warp takes a contiguous run of the list.
-__global__ void __launch_bounds__(WPB * 32) k_insert_left(Dev dp, const int *left, int items, RoundBuild B)
+// Insertions by one warp each: the staged Bowyer-Watson insertion, else split and flips, with
+// claims by compare-and-swap.  The points are those the rounds left out (a cavity above
+// their limits; left: the list), or one level of every instance (left null: positions
+// (2j + 1) 2^level, lvoff: its item offsets), for which the coarser levels are in already.
+// Each warp takes a contiguous run.
+__global__ void __launch_bounds__(WPB * 32) k_insert_warps(Dev dp, const int *left, int items, RoundBuild B, int level,
+                                                           const int *lvoff)
 {
     KD_BLOCK_DEV(dp);
     __shared__ WarpShared shs[WPB];
     int wib = threadIdx.x >> 5;
     int gw = blockIdx.x * (blockDim.x >> 5) + wib;
     int nw = gridDim.x * (blockDim.x >> 5);
-    Warp w = make_warp(&shs[wib], gw + 1, gw * 7 + 1315423911u, d);
+    Warp w = make_warp(&shs[wib], gw + 1, gw * 7 + (level + 1) * 1315423911u, d);
     const int per = (items + nw - 1) / nw;
     const int jend = min(items, (gw + 1) * per);
     for (int g = gw * per; g < jend; ++g) {
         if (read_status(d)) break;
-        const int item = __ldcg(left + g);
-        const int inst = B.ninst > 1 ? csr_find(B.pofs, B.ninst + 1, item) : 0;
+        int inst = 0, item;
+        if (left) {
+            item = __ldcg(left + g);
+            if (B.ninst > 1) inst = csr_find(B.pofs, B.ninst + 1, item);
+        } else {
+            if (B.ninst > 1) inst = csr_find(lvoff, B.ninst + 1, g);
+            const int k = B.ninst > 1 ? g - __ldg(lvoff + inst) : g;
+            item = __ldg(B.pofs + inst) + (int)((2ll * k + 1) << level);
+        }
         const int p0 = __ldg(B.pofs + inst), j = item - p0;
         const int v = __ldg(B.order + item);
         if (B.ninst > 1) set_instance(w, p0, __ldg(B.pofs + inst + 1) - p0);
