@@ -93,7 +93,7 @@ struct kdt {
     Buf key, bord, hist, hoff, exp_cnt, exp_off, exp_fill, exp_out, exp_rows;
     Buf btab, blev;  // batched build: per-instance tables, per-level item offsets
     // rounds (kdt_rounds.cuh): of a build, and of the steps (sized for mcap moves)
-    Buf rb_cnt, rb_lost, rb_hdr, rb_rec, rb_queue, rb_left;
+    Buf rb_cnt, rb_lost, rb_hdr, rb_rec, rb_queue, rb_left, rb_ref;
     Buf rm_cnt, rm_lost, rm_hdr, rm_rec, rm_slots, rm_left;
     int rm_rounds = 0, rm_ops = 0;
     int rm_layout = 0;  // rounds the counters have room for (a small step's too)
@@ -140,7 +140,7 @@ struct kdt {
     int tune_count = 0;
     double tune_ms[9] = {0};
     // host side
-    int *hscal = nullptr;  // pinned copy of the scalars (and two words more)
+    int *hscal = nullptr;  // pinned copy of the scalars (and four words more)
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr, ev3 = nullptr;
     kdt_stats stats{};
     // learned locate proposal and its training rows (kdt_mlp.cuh)
@@ -405,8 +405,9 @@ int certify_and_repair(kdt *h, bool full, int s0, int nslots, int wraps, int *de
 }
 
 // the counters of `rounds` rounds in one buffer: heads, offsets and losers (rounds + 1
-// entries each), the left list's length, the moves pending; `ops` operations a round
-size_t round_counter_ints(int rounds) { return 3 * (size_t)(rounds + 1) + 2; }
+// entries each), the lengths of the left and the refused list, the moves pending; `ops`
+// operations a round
+size_t round_counter_ints(int rounds) { return 3 * (size_t)(rounds + 1) + 3; }
 
 Rounds make_rounds(const Buf &cnt, int rounds, const Buf &lost, const Buf &hdr, const Buf &rec, int ops)
 {
@@ -416,13 +417,17 @@ Rounds make_rounds(const Buf &cnt, int rounds, const Buf &lost, const Buf &hdr, 
     R.off = c + (rounds + 1);
     R.lostcnt = c + 2 * (rounds + 1);
     R.left_count = c + 3 * (rounds + 1);
-    R.pending = R.left_count + 1;
+    R.refused_count = R.left_count + 1;
+    R.pending = R.left_count + 2;
     R.lost[0] = (int *)lost.p;
     R.lost[1] = (int *)lost.p + ops;
     R.hdr = (int4 *)hdr.p;
     R.rec = (int4 *)rec.p;
     R.slots = nullptr;
     R.left = nullptr;
+    R.refused = nullptr;
+    R.wide = nullptr;
+    R.nwide = 0;
     R.div = 0;
     R.few = 0;
     R.base = 0;
@@ -452,6 +457,17 @@ void launch_round(kdt *h, cudaStream_t st, const Dev &d, const Rounds &R, int b,
 // large ones their attempts.  1e6 points: 4 / 0 20.4 ms, 8 / 0 10.8, 12 / 0 9.8, 12 / 2048 9.7,
 // 12 / 8192 11.5, 16 / 4096 9.9 against 10.3 with 12 / 4096.
 constexpr int BUILD_DIV = 12, BUILD_FEW = 2048;
+// At least so many rounds between two looks at the counters.  What the rounds left out is
+// inserted there, while its cavities are as small as they will be: a dense row of 10,000
+// points facing 100 (degrees of 100 and more) took 2.6 s with all of it at the end, 50 ms so
+// (60-440 with one warp per insertion throughout); on a lattice of 300 x 300, one build in
+// ten left so many neighbouring points that their insertions ran out of retries.
+constexpr int BUILD_ROUNDS = 8;
+// Points in per warp that inserts what was left out: the cavities have more than 32 triangles,
+// and warps that meet lose their claims and leave edges to repair; fewer warps wait for one
+// another.  The rows 55 ms / 52 / 60 / 105, 3,000 rings of 60 points with a centre each 7.2 /
+// 6.8 / 8.5 / 800, with 64 / 128 / 512 / all points a warp.
+constexpr int LEFT_POINTS = 128;
 
 // One warp per insertion (k_insert_warps), at most `most` of them at once.
 void launch_insert_warps(kdt *h, const Dev &d, const int *left, int items, long long most, const RoundBuild &B,
@@ -486,7 +502,7 @@ int insert_levels(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
 
 // Insert every point of the instances whose first triangles are in (the points in Hilbert
 // order, the instances' levels in lv: ni + 1 item offsets per level, on the device at
-// dlv) in rounds, then what the rounds left with one warp per point.  Slots s0 ..
+// dlv) in rounds, and what the rounds leave out with one warp per point.  Slots s0 ..
 // s0 + nslots - 1 are the instances'.  Returns an ABI code.
 int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const int *dlv, int levels, int s0,
                   int nslots)
@@ -500,11 +516,12 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
     const int ops = (int)std::min<long long>(ROUND_OPS, std::max<long long>(64, std::max<long long>(np / BUILD_DIV, std::min<long long>(np, BUILD_FEW)) + 64));
     if (grow(h->rb_cnt, round_counter_ints(ROUND_MAX) * sizeof(int)) || grow(h->rb_lost, 2 * (size_t)ops * sizeof(int)) ||
         grow(h->rb_hdr, (size_t)ops * sizeof(int4)) || grow(h->rb_rec, (size_t)ops * 2 * RT * sizeof(int4)) ||
-        grow(h->rb_queue, (size_t)np * sizeof(int)) ||
-        grow(h->rb_left, (size_t)np * sizeof(int)))
+        grow(h->rb_queue, (size_t)np * sizeof(int)) || grow(h->rb_left, (size_t)np * sizeof(int)) ||
+        grow(h->rb_ref, (size_t)np * sizeof(int)))
         return KDT_ERR_CUDA;
     Rounds R = make_rounds(h->rb_cnt, ROUND_MAX, h->rb_lost, h->rb_hdr, h->rb_rec, ops);
     R.left = (int *)h->rb_left.p;
+    R.refused = (int *)h->rb_ref.p;
     R.div = BUILD_DIV;
     R.few = BUILD_FEW;
     R.base = 3 * ni;
@@ -522,44 +539,63 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
         h->stats.kernel_launches++;
         at += items;
     }
-    int b = 0;
     const RoundMoves M{nullptr};
-    long long in = R.base;  // points in at most
-    int batch = (int)(11.0 * std::log((double)np / ni)) + 4;
-    bool wide = false;
-    for (int pending = -1; b + batch <= ROUND_MAX;) {
-        for (int i = 0; i < batch; ++i, ++b) {
-            const long long most = std::min<long long>(
-                ops, std::max<long long>(64, std::max<long long>(in / BUILD_DIV, std::min<long long>(in, BUILD_FEW))));
-            launch_round<REGION_INSERT>(h, st, d, R, b, most, M, B, wide, false);
-            in = std::min(in + most, np);
+    auto left_warps = [ni](long long in) { return std::max<long long>(ni, in / LEFT_POINTS); };
+    int *hs = h->hscal + S_NUM;  // pinned: head, losers, left and refused so far
+    int b = 0, pend = B.total, nlost = 0, nleft = 0, nref = 0, left_done = 0, ref_done = 0;
+    long long in = R.base;  // points in, those left or refused among them
+    while (b < ROUND_MAX && (pend > 0 || nref > ref_done)) {
+        if (nleft > left_done) {
+            k_clear_owner<<<thread_grid(h, nslots, 256), 256, 0, st>>>(d.tn, s0, nslots);
+            launch_insert_warps(h, d, R.left + left_done, nleft - left_done, left_warps(in), B, 0, nullptr);
+            h->stats.kernel_launches++;
+            CK(cudaGetLastError());
+            int ds = 0;  // (the rounds' plans need every edge locally Delaunay)
+            if (certify_and_repair(h, true, s0, nslots, ni, &ds)) return KDT_ERR_CUDA;
+            if (ds) return dev_to_abi(ds);
+            left_done = nleft;
         }
-        h->stats.kernel_launches += 2 * batch;
+        int k = 0;
+        if (nref > ref_done && (pend == 0 || nref - ref_done >= std::max<long long>(8, in / 1024))) {
+            R.wide = R.refused + ref_done;
+            R.nwide = std::min(nref - ref_done, ops - nlost);
+            launch_round<REGION_INSERT>(h, st, d, R, b++, nlost + R.nwide, M, B, true, true);
+            ref_done += R.nwide;
+            pend += R.nwide;
+            R.nwide = 0;
+            ++k;
+        }
+        // rounds until the points in have grown fourfold, if every operation won
+        for (long long est = in; b < ROUND_MAX && (k < BUILD_ROUNDS || (est < 4 * in && est < np)); ++b, ++k) {
+            const long long most = std::min<long long>(
+                {(long long)ops, (long long)pend, std::max<long long>({64ll, est / BUILD_DIV, std::min<long long>(est, BUILD_FEW)})});
+            const bool wide = 32 * most <= (long long)ROUND_THREADS * 32 * sm_count(h->device);
+            launch_round<REGION_INSERT>(h, st, d, R, b, most, M, B, wide, wide);
+            est = std::min(est + most, np);
+        }
+        h->stats.kernel_launches += 2 * k;
         CK(cudaGetLastError());
-        int *hs = h->hscal + S_NUM;  // pinned
         CK(cudaMemcpyAsync(hs, R.head + b, sizeof(int), cudaMemcpyDeviceToHost, st));
         CK(cudaMemcpyAsync(hs + 1, R.lostcnt + b, sizeof(int), cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(hs + 2, R.left_count, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
         if (sync_scalars(h)) return KDT_ERR_CUDA;
         if (h->hscal[S_STATUS]) return dev_to_abi(h->hscal[S_STATUS]);
-        const int now = B.total - hs[0] + hs[1];
-        if (now == 0 || (wide && now == pending)) break;
-        // the rest in 32 lanes once it is small (what 16 cannot take is among it)
-        wide = wide || (hs[0] == B.total && now <= 4096);
-        pending = now;
-        batch = 8;
+        nlost = hs[1];
+        nleft = hs[2];
+        nref = hs[3];
+        pend = B.total - hs[0] + nlost;
+        in = R.base + hs[0] - nlost;
     }
     k_clear_owner<<<thread_grid(h, nslots, 256), 256, 0, st>>>(d.tn, s0, nslots);
-    k_build_rest<<<thread_grid(h, total, 256), 256, 0, st>>>(R, b, B);
-    h->stats.kernel_launches += 2;
-    CK(cudaMemcpyAsync(h->hscal + S_NUM, R.left_count, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    const int left = h->hscal[S_NUM];
-    if (left > 0) {
-        // about 16 triangles of room per concurrent insertion: more warps than that only
-        // collide on the same cavities (claims fail, back off, retry)
-        launch_insert_warps(h, d, R.left, left, std::max<long long>(8ll * ni, (np - left) / 8), B, 0, nullptr);
-        CK(cudaGetLastError());
+    h->stats.kernel_launches++;
+    if (pend > 0 || nref > ref_done) {  // (ROUND_MAX rounds)
+        k_build_rest<<<thread_grid(h, pend + nref - ref_done, 256), 256, 0, st>>>(R, b, B, R.refused + ref_done, nref - ref_done);
+        h->stats.kernel_launches++;
+        nleft += pend + nref - ref_done;
     }
+    if (nleft > left_done)
+        launch_insert_warps(h, d, R.left + left_done, nleft - left_done, left_warps(in), B, 0, nullptr);
+    CK(cudaGetLastError());
     if (sync_scalars(h)) return KDT_ERR_CUDA;
     return h->hscal[S_STATUS] ? dev_to_abi(h->hscal[S_STATUS]) : KDT_OK;
 }
@@ -920,7 +956,7 @@ void free_state(kdt *h)
     h->ppart = nullptr;
     h->mcap = 0; h->dirty_cap = 0; h->scan_tmp_cap = 0; h->rm_rounds = 0;
     Buf *bs[] = {&h->key, &h->bord, &h->hist, &h->hoff, &h->exp_cnt, &h->exp_off, &h->exp_fill, &h->exp_out, &h->exp_rows,
-                 &h->btab, &h->blev, &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left,
+                 &h->btab, &h->blev, &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left, &h->rb_ref,
                  &h->rm_cnt, &h->rm_lost, &h->rm_hdr, &h->rm_rec, &h->rm_slots, &h->rm_left,
                  &h->dc_dist, &h->dc_cmin, &h->dc_scal};
     for (Buf *b : bs) free_buf(*b);
@@ -1752,7 +1788,7 @@ int kdt_create(kdt **out, const kdt_config *cfg, int device, void *cuda_stream)
     h->cfg = c;
     if (cudaMalloc(&h->scal, S_NUM * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&h->counters, C_SLOTS * sizeof(unsigned long long)) != cudaSuccess ||
-        cudaMallocHost(&h->hscal, (S_NUM + 2) * sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&h->hscal, (S_NUM + 4) * sizeof(int)) != cudaSuccess ||
 
         cudaStreamCreateWithFlags(&h->cstream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreate(&h->ev0) != cudaSuccess || cudaEventCreate(&h->ev1) != cudaSuccess ||

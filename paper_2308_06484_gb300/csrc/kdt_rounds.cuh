@@ -68,6 +68,10 @@ struct Rounds {
     int *slots;     // moves only, per operation since the step's start: RT slots (-1: none)
     int *left;      // items for the warp-wide path
     int *left_count;
+    int *refused;   // builds: items 16 lanes could not plan, for a round of 32 lanes
+    int *refused_count;
+    const int *wide;  // builds: this round takes these nwide items (once refused) instead of fresh ones
+    int nwide;
     int *pending;   // moves only: moves not done after the last round
     int div;        // builds: operations up to the points inserted or up to `few`, and 1 / div of
                     // them beyond (0: no such limit)
@@ -76,7 +80,7 @@ struct Rounds {
     int ops;        // room for operations of one round
 };
 
-// the round's operations: losers, fresh items (total: length of the queue)
+// the round's operations: losers, then the wide list or fresh items (total: length of the queue)
 __device__ __forceinline__ void round_window(const Rounds &R, int b, int total, int &nlost, int &head, int &count)
 {
     nlost = __ldcg(R.lostcnt + b);
@@ -86,7 +90,7 @@ __device__ __forceinline__ void round_window(const Rounds &R, int b, int total, 
         const int in = R.base + head - nlost;
         lim = min(lim, max(max(64, in / R.div), min(in, R.few)));
     }
-    count = nlost + max(0, min(lim - nlost, total - head));
+    count = nlost + (R.nwide > 0 ? R.nwide : max(0, min(lim - nlost, total - head)));
 }
 
 // priority of operation x of round b: the round first, then a different order of the
@@ -143,8 +147,8 @@ __device__ __forceinline__ int near_start(const Dev &d, const int *order, int n,
 
 // RL lanes per operation.  With fewer operations than warps every operation has a warp to
 // itself, so no warp is as long as the union of two operations' paths.  An operation
-// outside RL's limits is planned again, by the 32-lane form when LAST is set or later, and
-// with LAST goes to the list of the warp-wide path.
+// outside RL's limits goes to the list of the warp-wide path when `last` is set; otherwise a
+// move is planned again in the next round and an insertion goes to the refused list.
 //
 // round_plan: `tid` of `nthreads` threads (whole warps), shared: one RegionShared per group of
 // the block.
@@ -158,7 +162,7 @@ __device__ __forceinline__ void round_plan(const Dev &d, const Rounds &R, int b,
     round_window(R, b, total, nlost, head, count);
     const int off = __ldcg(R.off + b);
     if (tid == 0) {
-        R.head[b + 1] = head + count - nlost;
+        R.head[b + 1] = R.nwide > 0 ? head : head + count - nlost;
         R.off[b + 1] = off + count;
     }
     constexpr int PER_WARP = 32 / RL;
@@ -171,7 +175,9 @@ __device__ __forceinline__ void round_plan(const Dev &d, const Rounds &R, int b,
     unsigned ex = 0, ti = 0, steps = 0;
     const int groups = alone ? warps : warps * PER_WARP;
     for (int x = alone ? tid / 32 : tid / RL; x < count; x += groups) {
-        const int item = x < nlost ? __ldcg(R.lost[b & 1] + x) : (MOVE ? head + x - nlost : __ldcg(B.queue + head + x - nlost));
+        const int item = x < nlost ? __ldcg(R.lost[b & 1] + x)
+                                   : (MOVE ? head + x - nlost
+                                           : __ldcg((R.nwide > 0 ? R.wide : B.queue + head) + x - nlost));
         RegionOut o;
         int4 *rec = R.rec + (size_t)x * (2 * RT);
         int rc, p;
@@ -201,7 +207,7 @@ __device__ __forceinline__ void round_plan(const Dev &d, const Rounds &R, int b,
         }
         ex += o.ex;
         ti += o.ti;
-        int nt = rc == RG_OK ? o.nt : (last ? -1 : 0);
+        int nt = rc == RG_OK ? o.nt : (last || !MOVE ? -1 : 0);
         if (rc == RG_VERTEX) {
             // q lies on a point: one that moves in this step may have left by the next round
             if (!MOVE) atomicCAS(d.status, 0, DEV_DUPLICATE);
@@ -215,7 +221,10 @@ __device__ __forceinline__ void round_plan(const Dev &d, const Rounds &R, int b,
         }
         if (l == 0) {
             steps += o.steps;
-            if (nt < 0) R.left[atomicAdd(R.left_count, 1)] = item;
+            if (nt < 0) {
+                if (MOVE || last) R.left[atomicAdd(R.left_count, 1)] = item;
+                else R.refused[atomicAdd(R.refused_count, 1)] = item;
+            }
             R.hdr[x] = make_int4(item, nt, pr, o.k | o.ncav << 8 | o.edge << 24 | o.ghost << 25 | o.prop << 26);
         }
         __syncwarp(gm);
@@ -449,13 +458,14 @@ __global__ void k_build_queue(RoundBuild B, const int *lvoff, int level, int ite
     }
 }
 
-// what is still to insert before round b (all of it when no round ran) to the list of the
+// what is still to insert before round b, `nref` refused items included, to the list of the
 // warp-wide path
-__global__ void k_build_rest(Rounds R, int b, RoundBuild B)
+__global__ void k_build_rest(Rounds R, int b, RoundBuild B, const int *refused, int nref)
 {
-    const int nlost = __ldcg(R.lostcnt + b), head = __ldcg(R.head + b);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nlost + B.total - head; i += gridDim.x * blockDim.x)
-        R.left[atomicAdd(R.left_count, 1)] = i < nlost ? __ldcg(R.lost[b & 1] + i) : __ldg(B.queue + head + i - nlost);
+    const int nlost = __ldcg(R.lostcnt + b), head = __ldcg(R.head + b), n = nlost + B.total - head;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n + nref; i += gridDim.x * blockDim.x)
+        R.left[atomicAdd(R.left_count, 1)] =
+            i < nlost ? __ldcg(R.lost[b & 1] + i) : (i < n ? __ldg(B.queue + head + i - nlost) : __ldcg(refused + i - n));
 }
 
 // Insertions by one warp each: the staged Bowyer-Watson insertion, else split and flips, with

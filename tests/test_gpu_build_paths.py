@@ -33,3 +33,58 @@ def test_build_warps_batch():
     for i, xy in enumerate(sets):
         assert_same(t.export_triangles_inst(i), xy, "instance %d" % i)
     assert t.verify() == 0
+
+
+def _rows(dense, sparse, bits):
+    """A dense row of points facing a sparse one: the sparse points' degrees are
+    dense / sparse, and each of them is inserted into a cavity of that size."""
+    L = 1 << bits
+    d = np.stack([np.linspace(0, L - 1, dense).astype(np.int64), np.full(dense, L // 2)], 1)
+    s = np.stack([np.linspace(0, L - 1, sparse).astype(np.int64), np.full(sparse, L // 2 + L // (4 * sparse))], 1)
+    return np.concatenate([d, s]).astype(np.int32)
+
+
+@pytest.mark.parametrize("dense,sparse", [(2000, 20), (10000, 100), (20000, 1000)])
+def test_rows_of_unlike_density(dense, sparse):
+    """Points the rounds cannot take are inserted while their cavities are small: put off to
+    the end they cost walks of thousands of steps (2,800 per point) and repairs of as many
+    flips."""
+    xy = _rows(dense, sparse, 26)
+    t = _tri(domain_bits=26)
+    t.build(xy)
+    st = t.stats()
+    assert t.verify() == 0
+    assert_same(t.export_triangles(), xy, "rows %d / %d" % (dense, sparse))
+    assert st["walk_steps"] < 100 * len(xy)
+    assert st["fixup_flips"] < 20 * len(xy)
+
+
+def test_many_refused_insertions():
+    """12,000 rings of 40 points with a centre each: more insertions than 4,096 have a cavity
+    beyond 16 lanes.  A build of uniform points takes some 300 launches."""
+    k, nr, bits = 40, 12000, 26
+    L, g = 1 << bits, 110
+    c = L // g
+    a = 2 * np.pi * np.arange(k) / k
+    base = np.rint(np.stack([0.4 * c * np.cos(a), 0.4 * c * np.sin(a)], 1)).astype(np.int64)
+    base = np.concatenate([[[0, 0]], base])
+    i = np.arange(nr)
+    at = np.stack([(i % g) * c + c // 2, (i // g) * c + c // 2], 1)
+    xy = (base[None] + at[:, None]).reshape(-1, 2)
+    xy = np.ascontiguousarray(xy[np.random.default_rng(1).permutation(len(xy))].astype(np.int32))
+    t = _tri(domain_bits=bits)
+    t.build(xy)
+    assert t.verify() == 0
+    assert t.stats()["kernel_launches"] < 1500
+
+
+def test_lattice_builds():
+    """A lattice (every square's corners cocircular), built often: the order in which
+    insertions meet differs from build to build."""
+    a = np.arange(300)
+    xy = np.ascontiguousarray((np.stack(np.meshgrid(a, a), -1).reshape(-1, 2) * 7).astype(np.int32))
+    t = _tri(domain_bits=20)
+    for _ in range(50):
+        t.build(xy)
+    assert t.verify() == 0
+    assert_same(t.export_triangles(), xy, "lattice")
