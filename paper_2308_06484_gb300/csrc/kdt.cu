@@ -483,17 +483,24 @@ void launch_insert_warps(kdt *h, const Dev &d, const int *left, int items, long 
     h->stats.kernel_launches++;
 }
 
-// Insert every point with kdt_config.build_warps warps, level by level (a level once the
-// coarser ones are in: its walks start next to their points and its cavities are small and
-// apart; 20,000 points with 64 warps 10.8 ms, all levels at once from the first triangle
-// 29.8 ms, and with 1,000 warps the retries ran out).
+// Builds of so many levels at most (up to 8 points, up to 4 in each instance of a batch) go
+// level by level: a round's chain and the counters' way to the host are longer than a launch
+// a level.  3 points 112 us against 194 in rounds, 8 points 219 and 229, 16 points 326 and 372;
+// 8 instances of 4 points 155 and 231, of 10 points 431 and 302.
+constexpr int TINY_LEVELS = 3, TINY_LEVELS_BATCH = 2;
+
+// Insert every point with kdt_config.build_warps warps (8 an instance where that is 0), level
+// by level (a level once the coarser ones are in: its walks start next to their points and
+// its cavities are small and apart; 20,000 points with 64 warps 10.1 ms, all levels at once
+// from the first triangle 26 ms, and with 1,000 warps the retries ran out).
 int insert_levels(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const int *dlv, int levels)
 {
     const int ni = B.ninst;
     for (int l = levels - 1; l >= 0; --l) {
         const int items = lv[(size_t)l * (ni + 1) + ni];
         if (items <= 0) continue;
-        launch_insert_warps(h, d, nullptr, items, h->cfg.build_warps, B, l, dlv ? dlv + (size_t)l * (ni + 1) : nullptr);
+        launch_insert_warps(h, d, nullptr, items, h->cfg.build_warps > 0 ? h->cfg.build_warps : 8ll * ni, B, l,
+                            dlv ? dlv + (size_t)l * (ni + 1) : nullptr);
         CK(cudaGetLastError());
     }
     if (sync_scalars(h)) return KDT_ERR_CUDA;
@@ -507,7 +514,8 @@ int insert_levels(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
 int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const int *dlv, int levels, int s0,
                   int nslots)
 {
-    if (h->cfg.build_warps > 0) return insert_levels(h, d, B, lv, dlv, levels);
+    if (h->cfg.build_warps > 0 || levels <= (B.ninst > 1 ? TINY_LEVELS_BATCH : TINY_LEVELS))
+        return insert_levels(h, d, B, lv, dlv, levels);
     cudaStream_t st = h->stream;
     const int ni = B.ninst;
     long long total = 0;

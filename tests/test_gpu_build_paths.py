@@ -88,3 +88,31 @@ def test_lattice_builds():
         t.build(xy)
     assert t.verify() == 0
     assert_same(t.export_triangles(), xy, "lattice")
+
+
+@pytest.mark.parametrize("n", list(range(3, 35)))
+def test_small_builds(n):
+    """Around the sizes where a build changes from levels to rounds; a handful of points takes
+    a launch a level (47 launches in rounds)."""
+    t = _tri(domain_bits=16)
+    for seed in range(4):
+        xy = W.uniform_points(n, 16, 100 * n + seed)
+        before = t.stats()["kernel_launches"]
+        t.build(xy)
+        launches = t.stats()["kernel_launches"] - before
+        assert_same(t.export_triangles(), xy, "%d points" % n)
+        if n <= 8:
+            assert launches <= 20
+    assert t.verify() == 0
+
+
+@pytest.mark.parametrize("n,instances", [(3, 5), (4, 300), (5, 40), (8, 40), (9, 40)])
+def test_small_instances(n, instances):
+    sets = [W.uniform_points(n, 12, i) for i in range(instances)]
+    t = _tri(domain_bits=12)
+    t.build_batch(sets)
+    if n <= 4:
+        assert t.stats()["kernel_launches"] <= 20
+    for i in range(0, instances, 7):
+        assert_same(t.export_triangles_inst(i), sets[i], "instance %d" % i)
+    assert t.verify() == 0
