@@ -700,8 +700,9 @@ int rebuild_batch(kdt *h)
     CK(cudaMemcpyAsync(bbox, hb.data(), hb.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(h->tri, 0, 2 * (size_t)h->cap * sizeof(int4), st));
     k_fill_int<<<thread_grid(h, n, 256), 256, 0, st>>>(h->pt_tri, n, -1);
-    k_range_batch<<<thread_grid(h, (n + 31) / 32, 256), 256, 0, st>>>(h->xy, n, h->d_pofs, ni, h->cfg.domain_bits,
-                                                          h->scal + S_STATUS, bbox);
+    const int run = std::min(RANGE_RUN, std::max(32, n / (8 * sm_count(h->device))));
+    k_range_batch<<<thread_grid(h, 32ll * ((n + run - 1) / run), 256), 256, 0, st>>>(
+        h->xy, n, h->d_pofs, ni, h->cfg.domain_bits, h->scal + S_STATUS, bbox, run);
     h->stats.kernel_launches += 2;
     CK(cudaMemcpyAsync(hb.data(), bbox, hb.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
     if (sync_scalars(h)) return KDT_ERR_CUDA;

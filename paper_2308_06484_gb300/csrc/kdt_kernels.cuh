@@ -1038,7 +1038,9 @@ __global__ void k_init(Dev d, const int *order, const int *third, int *tri_count
 // over all instances (kdt_rounds.cuh), level by level.
 
 // bounding box of every instance (bbox[4 i .. 4 i + 3]) and the range check: a warp takes a
-// run of RANGE_RUN points and, while they are of one instance, keeps its box in registers
+// run of points and, while they are of one instance, keeps its box in registers.  The run
+// is RANGE_RUN points, shorter (32 at least) where that gives too few warps: 512 instances of
+// 4 points were two warps' work, each instance's box after the other's.
 constexpr int RANGE_RUN = 1024;
 
 __device__ __forceinline__ void range_flush(int *b, int mnx, int mny, int mxx, int mxy)
@@ -1055,12 +1057,13 @@ __device__ __forceinline__ void range_flush(int *b, int mnx, int mny, int mxx, i
     }
 }
 
-__global__ void k_range_batch(const int2 *xy, int n, const int *pofs, int ninst, int bits, int *status, int *bbox)
+__global__ void k_range_batch(const int2 *xy, int n, const int *pofs, int ninst, int bits, int *status, int *bbox,
+                              int len)
 {
     const long long lim = 1ll << bits;
     const int lane = threadIdx.x & 31, warps = gridDim.x * (blockDim.x >> 5);
-    for (int run = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); (long long)run * RANGE_RUN < n; run += warps) {
-        const int lo = run * RANGE_RUN, hi = min(n, lo + RANGE_RUN);
+    for (int run = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); (long long)run * len < n; run += warps) {
+        const int lo = run * len, hi = min(n, lo + len);
         int inst = csr_find(pofs, ninst + 1, lo);
         for (int i0 = lo; i0 < hi;) {
             // the part of the run that is this instance's

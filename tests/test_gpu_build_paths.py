@@ -116,3 +116,26 @@ def test_small_instances(n, instances):
     for i in range(0, instances, 7):
         assert_same(t.export_triangles_inst(i), sets[i], "instance %d" % i)
     assert t.verify() == 0
+
+
+@pytest.mark.parametrize("n", [64, 40000, 52000, 1300000])
+def test_boxes_of_uneven_instances(n):
+    """Instances that begin and end anywhere in the runs of points a warp takes for the bounding
+    boxes (runs of 32 to 1,024 points); a point out of range anywhere is refused."""
+    from paper_2308_06484_gb300 import kdt
+    rng = np.random.default_rng(n)
+    cuts = np.unique(np.concatenate([[0, n], 3 + rng.integers(0, n - 6, size=min(300, n // 16))]))
+    sizes = np.diff(cuts)
+    sizes = sizes[sizes >= 3]
+    sets = [W.uniform_points(int(k), 20, i) // (1 + i % 5) for i, k in enumerate(sizes)]
+    sets = [np.ascontiguousarray(s[np.sort(np.unique(s, axis=0, return_index=True)[1])]) for s in sets]
+    t = _tri(domain_bits=20)
+    t.build_batch(sets)
+    assert t.verify() == 0
+    for i in range(0, len(sets), 1 + len(sets) // 5):
+        if len(sets[i]) < 20000:
+            assert_same(t.export_triangles_inst(i), sets[i], "instance %d" % i)
+    bad = [s.copy() for s in sets]
+    bad[-1][-1] = (1 << 20, 5)
+    with pytest.raises(kdt.KDTError):
+        t.build_batch(bad)
