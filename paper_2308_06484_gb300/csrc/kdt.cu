@@ -483,11 +483,11 @@ void launch_insert_warps(kdt *h, const Dev &d, const int *left, int items, long 
     h->stats.kernel_launches++;
 }
 
-// Builds of so many levels at most (up to 8 points, up to 4 in each instance of a batch) go
+// Builds of so many levels at most (up to 16 points, up to 4 in each instance of a batch) go
 // level by level: a round's chain and the counters' way to the host are longer than a launch
-// a level.  3 points 112 us against 194 in rounds, 8 points 219 and 229, 16 points 326 and 372;
-// 8 instances of 4 points 155 and 231, of 10 points 431 and 302.
-constexpr int TINY_LEVELS = 3, TINY_LEVELS_BATCH = 2;
+// a level.  3 points 112 us against 194 in rounds, 8 points 219 and 229, 16 points 326 and
+// 372, 24 points 514 and 429; 8 instances of 4 points 155 and 231, of 10 points 431 and 302.
+constexpr int TINY_LEVELS = 4, TINY_LEVELS_BATCH = 2;
 
 // Insert every point with kdt_config.build_warps warps (8 an instance where that is 0), level
 // by level (a level once the coarser ones are in: its walks start next to their points and

@@ -101,7 +101,7 @@ def test_small_builds(n):
         t.build(xy)
         launches = t.stats()["kernel_launches"] - before
         assert_same(t.export_triangles(), xy, "%d points" % n)
-        if n <= 8:
+        if n <= 16:
             assert launches <= 20
     assert t.verify() == 0
 
