@@ -43,6 +43,40 @@ constexpr int TUNE_PPP[3] = {128, 256, 512};
 constexpr int TUNE_WPP[3] = {1, 2, 4};
 constexpr int TUNE_STEPS = 1;  // timed steps per configuration
 
+// Rounds of a step beyond those that take every move once: the losers of the first are
+// few (one in 250 at one move per 250 uniform points, one in three where most points of
+// sparse cells move), those of the next fewer; the last ones go to the kinetic kernel.
+// An empty round costs about 5 us (4 more on 1e6 points: 85 -> 120 us a step), a round more
+// on 16e6 clustered points saves 30 us (2 rounds 1.55, 4 1.47, 6 1.43 ms), on 512 instances
+// it costs 20.
+constexpr int STEP_EXTRA_ROUNDS = 2, STEP_EXTRA_ROUNDS_MANY = 4, STEP_MANY = 32768;
+
+// A step's class, by its own number of moves: up to 2,048, 8,192, STEP_MANY - 1, then ROUND_OPS
+// times a power of two.  It gives the rounds launched and the grids, and each class has a
+// graph of its own, so one large step makes no later one longer (2,000 moves among 3e6
+// points 65 us, 338 after a step of all points when the largest step so far decided; among
+// 2e5 points 77, after one of 40,000 137 then, 91 with one class below STEP_MANY).
+constexpr int STEP_CLASSES = 16, STEP_MANY_CLASS = 3;
+constexpr int SMALL_GRAPH = STEP_CLASSES, STEP_GRAPHS = STEP_CLASSES + 1;
+
+constexpr long long class_moves(int c)
+{
+    return c < STEP_MANY_CLASS ? std::min(2048ll << 2 * c, STEP_MANY - 1ll) : (long long)ROUND_OPS << (c - STEP_MANY_CLASS);
+}
+
+int step_class(long long m)
+{
+    int c = 0;
+    while (class_moves(c) < m) ++c;
+    return c;
+}
+
+int class_rounds(int c)
+{
+    return c < STEP_MANY_CLASS ? 1 + STEP_EXTRA_ROUNDS : (1 << (c - STEP_MANY_CLASS)) + STEP_EXTRA_ROUNDS_MANY;
+}
+static_assert(class_moves(STEP_CLASSES - 1) >= 1ll << 30, "a class for every step");
+
 }  // namespace
 
 struct kdt {
@@ -92,11 +126,11 @@ struct kdt {
     // build / export temporaries (kept between calls)
     Buf key, bord, hist, hoff, exp_cnt, exp_off, exp_fill, exp_out, exp_rows;
     Buf btab, blev;  // batched build: per-instance tables, per-level item offsets
-    // rounds (kdt_rounds.cuh): of a build, and of the steps (sized for mcap moves)
+    // rounds (kdt_rounds.cuh): of a build, and of the steps
     Buf rb_cnt, rb_lost, rb_hdr, rb_rec, rb_queue, rb_left, rb_ref;
     Buf rm_cnt, rm_lost, rm_hdr, rm_rec, rm_slots, rm_left;
-    int rm_rounds = 0, rm_ops = 0;
-    int rm_layout = 0;  // rounds the counters have room for (a small step's too)
+    int rm_cap = 0, rm_ops = 0;  // moves of a step, operations of a round they have room for
+    int rm_layout = 0;           // rounds the counters have room for (a small step's too)
     // d-calculation: results, running minimum (per N)
     Buf dc_dist, dc_cmin, dc_scal;
     int64_t d2_run = INT64_MAX;
@@ -128,11 +162,11 @@ struct kdt {
     int *ctl = nullptr;   // device
     int *hctl = nullptr;  // pinned host
     cudaStream_t cstream = nullptr;
-    // [0]: the step's graph, [1]: a small step's (k_step_small), and the buffer generation
-    // each was captured for
-    cudaGraph_t graph[2] = {nullptr, nullptr};
-    cudaGraphExec_t gexec[2] = {nullptr, nullptr};
-    int graph_gen[2] = {-1, -1};
+    // the graphs of the steps' classes (step_class), of a small step (k_step_small) last, and the
+    // buffer generation each was captured for
+    cudaGraph_t graph[STEP_GRAPHS] = {};
+    cudaGraphExec_t gexec[STEP_GRAPHS] = {};
+    int graph_gen[STEP_GRAPHS] = {};
     int gen = 0;         // bumped whenever step buffers or tables change
     // autotuner state: configuration index being timed, accumulated times
     int tune_idx = -1;
@@ -803,19 +837,11 @@ int ensure_moves(kdt *h, int64_t m)
     if (dc > (1ll << 30)) dc = 1ll << 30;
     if (dalloc(&h->dirty, (size_t)dc)) return KDT_ERR_CUDA;
     h->dirty_cap = (int)dc;
-    h->rm_rounds = 0;  // (ensure_rounds sizes them again)
     h->gen++;
     return 0;
 }
 
-// Rounds of a step beyond those that take every move once: the losers of the first are
-// few (one in 250 at one move per 250 uniform points, one in three where most points of
-// sparse cells move), those of the next fewer; the last ones go to the kinetic kernel.
-// An empty round costs about 5 us (4 more on 1e6 points: 85 -> 120 us a step), a round more
-// on 16e6 clustered points saves 30 us (2 rounds 1.55, 4 1.47, 6 1.43 ms), on 512 instances
-// it costs 20.
 constexpr int FEW_LEFT = 1024;  // moves the kinetic kernel takes as a list, a warp each
-constexpr int STEP_EXTRA_ROUNDS = 2, STEP_EXTRA_ROUNDS_MANY = 4, STEP_MANY = 32768;
 
 // Do the step's moves go through rounds?  The paper's method (delete and insert), without
 // training rows and with no proposal or one the planner evaluates; else the kinetic kernel
@@ -826,19 +852,19 @@ bool step_in_rounds(const kdt *h)
            h->cfg.kinetic_warps == 0;
 }
 
-int ensure_rounds(kdt *h)
+// Room for the rounds of a step of m moves.
+int ensure_rounds(kdt *h, int64_t m)
 {
-    if (h->rm_rounds > 0) return 0;
-    const int ops = std::min(h->mcap, ROUND_OPS);
-    const int rounds =
-        (h->mcap + ops - 1) / ops + (h->mcap >= STEP_MANY ? STEP_EXTRA_ROUNDS_MANY : STEP_EXTRA_ROUNDS);
-    const int layout = std::max(rounds, SMALL_ROUNDS);
+    if (m <= h->rm_cap) return 0;
+    const int cap = (int)std::max<int64_t>(m, 1024), ops = std::min(cap, ROUND_OPS);
+    const int rounds = class_rounds(step_class(cap)), layout = std::max(rounds, SMALL_ROUNDS);
     if (grow(h->rm_cnt, round_counter_ints(layout) * sizeof(int)) || grow(h->rm_lost, 2 * (size_t)ops * sizeof(int)) ||
         grow(h->rm_hdr, (size_t)ops * sizeof(int4)) || grow(h->rm_rec, (size_t)ops * 2 * RT * sizeof(int4)) ||
-        grow(h->rm_slots, std::max((size_t)rounds * ops, (size_t)SMALL_ROUNDS * SMALL_MOVES) * RT * sizeof(int)) || grow(h->rm_left, (size_t)h->mcap * sizeof(int)))
+        grow(h->rm_slots, std::max((size_t)rounds * ops, (size_t)SMALL_ROUNDS * SMALL_MOVES) * RT * sizeof(int)) ||
+        grow(h->rm_left, (size_t)cap * sizeof(int)))
         return KDT_ERR_CUDA;
     h->rm_ops = ops;
-    h->rm_rounds = rounds;
+    h->rm_cap = cap;
     h->rm_layout = layout;
     h->gen++;
     return 0;
@@ -923,8 +949,7 @@ void free_quadtree(kdt *h)
 // No triangulation any more, the arrays kept for the next build.
 void reset_state(kdt *h)
 {
-    drop_graph(h, 0);
-    drop_graph(h, 1);
+    for (int g = 0; g < STEP_GRAPHS; ++g) drop_graph(h, g);
     h->gen++;
     free_quadtree(h);
     h->dloc_valid = false;
@@ -963,7 +988,7 @@ void free_state(kdt *h)
     h->pguess = nullptr;
     h->pfeat = nullptr;
     h->ppart = nullptr;
-    h->mcap = 0; h->dirty_cap = 0; h->scan_tmp_cap = 0; h->rm_rounds = 0;
+    h->mcap = 0; h->dirty_cap = 0; h->scan_tmp_cap = 0; h->rm_cap = 0;
     Buf *bs[] = {&h->key, &h->bord, &h->hist, &h->hoff, &h->exp_cnt, &h->exp_off, &h->exp_fill, &h->exp_out, &h->exp_rows,
                  &h->btab, &h->blev, &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left, &h->rb_ref,
                  &h->rm_cnt, &h->rm_lost, &h->rm_hdr, &h->rm_rec, &h->rm_slots, &h->rm_left,
@@ -1171,14 +1196,15 @@ int tc_grid(const kdt *h, long long rows)
     return (int)std::min<long long>(tiles, 3ll * sm_count(h->device));
 }
 
-int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, bool from_ctl, bool small)
+int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, bool from_ctl, int which)
 {
-    int cap = from_ctl ? h->mcap : mi;
+    const bool rounds = step_in_rounds(h), small = which == SMALL_GRAPH;
+    const int nrounds = small ? SMALL_ROUNDS : class_rounds(which);
+    const int cap = !from_ctl ? mi : (rounds && !small ? (int)std::min<long long>(h->mcap, class_moves(which)) : h->mcap);
     Inst I = make_inst(h);
     // the step's control words and move offsets, from pinned host memory (a captured
     // copy reads them when the graph runs)
     CK(cudaMemcpyAsync(h->ctl, h->hctl, (4 + h->ninst + 1) * sizeof(int), cudaMemcpyHostToDevice, st));
-    const bool rounds = step_in_rounds(h);
     const unsigned evflags0 = from_ctl ? cudaEventRecordExternal : cudaEventRecordDefault;
     Rounds R{};
     if (rounds) {
@@ -1252,11 +1278,10 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
         const RoundMoves M{h->gmoves};
         const RoundBuild B{nullptr, nullptr, nullptr, nullptr, nullptr, 0, mi, 0};
         auto launch_moves = d.pguess ? launch_round<REGION_GUESS> : launch_round<REGION_MOVE>;
-        for (int b = 0; b < h->rm_rounds; ++b)
-            launch_moves(h, st, d, R, b, std::min(cap, h->rm_ops), M, B, b + 1 == h->rm_rounds,
-                         b + 1 == h->rm_rounds);
+        for (int b = 0; b < nrounds; ++b)
+            launch_moves(h, st, d, R, b, std::min(cap, h->rm_ops), M, B, b + 1 == nrounds, b + 1 == nrounds);
         k_round_clear<<<thread_grid(h, (long long)cap * (RT / 4), 256), 256, 0, st>>>(
-            d, R, h->rm_rounds, mi, I, h->cfg.domain_bits, h->gmoves, h->old_xy, h->head, h->next);
+            d, R, nrounds, mi, I, h->cfg.domain_bits, h->gmoves, h->old_xy, h->head, h->next);
     }
     return enqueue_kinetic(h, st, d, I, from_ctl, h->mcap);
 }
@@ -1403,7 +1428,7 @@ int step_core(kdt *h, const kdt_move *moves, const int64_t *moff, int64_t m)
     if (rc) return rc;
     rc = ensure_big(h);
     if (rc) return rc;
-    if (step_in_rounds(h)) rc = ensure_rounds(h);
+    if (step_in_rounds(h)) rc = ensure_rounds(h, m);
     if (rc) return rc;
     if (h->qhist && h->scan_tmp_cap < (h->qF * h->qF + SCAN_TILE - 1) / SCAN_TILE + 1) {
         // the step graph scans every fine cell: its scan scratch must exist before capture
@@ -1422,15 +1447,15 @@ int step_core(kdt *h, const kdt_move *moves, const int64_t *moff, int64_t m)
     bool timed = h->cfg.timing || (h->tune_idx >= 0 && !h->tune_done);
     const bool rounds = step_in_rounds(h);
     const bool small = rounds && m <= SMALL_MOVES && h->cfg.plan == 0 && !h->qhist && h->ncells_cap <= SMALL_CELLS;
-    const int which = small ? 1 : 0;
+    const int which = small ? SMALL_GRAPH : (rounds ? step_class(m) : 0);
     if (h->cfg.use_graph) {
         // one graph launch per step
-        if (h->graph_gen[which] != h->gen) {
+        if (!h->gexec[which] || h->graph_gen[which] != h->gen) {
             drop_graph(h, which);
             Dev dg = d;
             dg.ctl = h->ctl;
             CK(cudaStreamBeginCapture(h->cstream, cudaStreamCaptureModeThreadLocal));
-            int er = enqueue_step(h, h->cstream, dg, nullptr, 0, true, small);
+            int er = enqueue_step(h, h->cstream, dg, nullptr, 0, true, which);
             cudaGraph_t g = nullptr;
             cudaError_t ce = cudaStreamEndCapture(h->cstream, &g);
             if (er || ce != cudaSuccess) {
@@ -1451,13 +1476,13 @@ int step_core(kdt *h, const kdt_move *moves, const int64_t *moff, int64_t m)
         if (timed) CK(cudaEventRecord(h->ev3, st));
     } else {
         if (timed) CK(cudaEventRecord(h->ev2, st));
-        if (enqueue_step(h, st, d, mp, mi, false, small)) return KDT_ERR_CUDA;
+        if (enqueue_step(h, st, d, mp, mi, false, which)) return KDT_ERR_CUDA;
         if (timed) CK(cudaEventRecord(h->ev3, st));
     }
     h->stats.kernel_launches += small ? 3 : 4 + ((h->cfg.plan & PLAN_ORDER) ? 2 : 0) +
                                 ((h->cfg.plan & PLAN_ORDER) || (h->prop_on && (h->cfg.plan & PLAN_NETWORK)) ? 1 : 0) +
                                 (h->prop_on && (h->cfg.plan & PLAN_NETWORK) && (h->cfg.plan & PLAN_TENSOR) ? 1 : 0) +
-                                (h->qhist ? h->qD + 5 : 0) + (rounds ? 2 * h->rm_rounds + 1 : 0);
+                                (h->qhist ? h->qD + 5 : 0) + (rounds ? 2 * class_rounds(which) + 1 : 0);
     CK(cudaStreamSynchronize(st));
     if (h->qhist) h->ncells = h->qleaves = h->hscal[S_NCELLS];
     if (timed) {
