@@ -128,7 +128,7 @@ struct kdt {
     Buf btab, blev;  // batched build: per-instance tables, per-level item offsets
     // rounds (kdt_rounds.cuh): of a build, and of the steps
     Buf rb_cnt, rb_lost, rb_hdr, rb_rec, rb_queue, rb_left, rb_ref;
-    Buf rm_cnt, rm_lost, rm_hdr, rm_rec, rm_slots, rm_left;
+    Buf rm_cnt, rm_lost, rm_hdr, rm_rec, rm_slots, rm_left, rm_ref;
     int rm_cap = 0, rm_ops = 0;  // moves of a step, operations of a round they have room for
     int rm_layout = 0;           // rounds the counters have room for (a small step's too)
     // d-calculation: results, running minimum (per N)
@@ -861,7 +861,7 @@ int ensure_rounds(kdt *h, int64_t m)
     if (grow(h->rm_cnt, round_counter_ints(layout) * sizeof(int)) || grow(h->rm_lost, 2 * (size_t)ops * sizeof(int)) ||
         grow(h->rm_hdr, (size_t)ops * sizeof(int4)) || grow(h->rm_rec, (size_t)ops * 2 * RT * sizeof(int4)) ||
         grow(h->rm_slots, std::max((size_t)rounds * ops, (size_t)SMALL_ROUNDS * SMALL_MOVES) * RT * sizeof(int)) ||
-        grow(h->rm_left, (size_t)cap * sizeof(int)))
+        grow(h->rm_left, (size_t)cap * sizeof(int)) || grow(h->rm_ref, (size_t)cap * sizeof(int)))
         return KDT_ERR_CUDA;
     h->rm_ops = ops;
     h->rm_cap = cap;
@@ -991,7 +991,7 @@ void free_state(kdt *h)
     h->mcap = 0; h->dirty_cap = 0; h->scan_tmp_cap = 0; h->rm_cap = 0;
     Buf *bs[] = {&h->key, &h->bord, &h->hist, &h->hoff, &h->exp_cnt, &h->exp_off, &h->exp_fill, &h->exp_out, &h->exp_rows,
                  &h->btab, &h->blev, &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left, &h->rb_ref,
-                 &h->rm_cnt, &h->rm_lost, &h->rm_hdr, &h->rm_rec, &h->rm_slots, &h->rm_left,
+                 &h->rm_cnt, &h->rm_lost, &h->rm_hdr, &h->rm_rec, &h->rm_slots, &h->rm_left, &h->rm_ref,
                  &h->dc_dist, &h->dc_cmin, &h->dc_scal};
     for (Buf *b : bs) free_buf(*b);
 }
@@ -1211,6 +1211,8 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
         R = make_rounds(h->rm_cnt, h->rm_layout, h->rm_lost, h->rm_hdr, h->rm_rec, h->rm_ops);
         R.slots = (int *)h->rm_slots.p;
         R.left = (int *)h->rm_left.p;
+        R.refused = (int *)h->rm_ref.p;
+        R.wide = R.refused;
         I.pending = R.pending;
         I.left = R.left;
         I.few_left = std::min(FEW_LEFT, h->mcap / 4);  // (each can be left for later DQ_PASSES times)
@@ -1278,8 +1280,11 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
         const RoundMoves M{h->gmoves};
         const RoundBuild B{nullptr, nullptr, nullptr, nullptr, nullptr, 0, mi, 0};
         auto launch_moves = d.pguess ? launch_round<REGION_GUESS> : launch_round<REGION_MOVE>;
-        for (int b = 0; b < nrounds; ++b)
-            launch_moves(h, st, d, R, b, std::min(cap, h->rm_ops), M, B, b + 1 == nrounds, b + 1 == nrounds);
+        for (int b = 0; b < nrounds; ++b) {
+            const bool last = b + 1 == nrounds;
+            R.nwide = last ? -1 : 0;
+            launch_moves(h, st, d, R, b, std::min(cap, h->rm_ops), M, B, last, last);
+        }
         k_round_clear<<<thread_grid(h, (long long)cap * (RT / 4), 256), 256, 0, st>>>(
             d, R, nrounds, mi, I, h->cfg.domain_bits, h->gmoves, h->old_xy, h->head, h->next);
     }

@@ -40,7 +40,8 @@ constexpr int RT = 32;     // most triangles an operation writes
 constexpr int RWALK = 1 << 12;  // steps of a walk before the operation is left to the other path
 
 enum RegionMode : int { REGION_INSERT = 0, REGION_MOVE = 1, REGION_GUESS = 2 };
-enum RegionResult : int { RG_OK = 0, RG_BAIL = 1, RG_VERTEX = 2 };
+// RG_BAIL: outside the limits of RL lanes, RG_LEFT: of any number of lanes
+enum RegionResult : int { RG_OK = 0, RG_BAIL = 1, RG_VERTEX = 2, RG_LEFT = 3 };
 
 // What the RL lanes of an operation share (RL: also the largest degree, cavity and border).
 template <int RL>
@@ -186,7 +187,7 @@ __device__ __forceinline__ int region_plan(const D &d, RegionShared<RL> &sh, int
             // nothing but that line (the other path decides)
             const int g = __ffs((int)gh) - 1, f0 = g + 1 < k ? g + 1 : 0, f1 = f0 + 1 < k ? f0 + 1 : 0;
             const int2 x0 = sh2(x, f0), x1 = sh2(x, f1);
-            if (!votes(inl && id >= 0 && orient2d(x0, x1, x) != 0)) return RG_BAIL;
+            if (!votes(inl && id >= 0 && orient2d(x0, x1, x) != 0)) return RG_LEFT;
         }
         // ---- 1. delete: ears
         unsigned alive = 0xffffffffu >> (32 - k);
@@ -326,7 +327,8 @@ __device__ __forceinline__ int region_plan(const D &d, RegionShared<RL> &sh, int
         // ---- visibility walk (exact orientations; the triangulation is Delaunay, so it ends)
         int t = start;
         while (true) {
-            if (t < 0 || t >= d.cap || ++o.steps > RWALK) return RG_BAIL;
+            if (t < 0 || t >= d.cap) return RG_BAIL;
+            if (++o.steps > RWALK) return RG_LEFT;
             const int4 v = __ldcg(d.tv + t), n = __ldcg(d.tn + t);
             if (!(v.w & 1)) return RG_BAIL;
             const int2 a = v.x >= 0 ? __ldcg(d.xy + v.x) : zero, b = v.y >= 0 ? __ldcg(d.xy + v.y) : zero,

@@ -68,10 +68,10 @@ struct Rounds {
     int *slots;     // moves only, per operation since the step's start: RT slots (-1: none)
     int *left;      // items for the warp-wide path
     int *left_count;
-    int *refused;   // builds: items 16 lanes could not plan, for a round of 32 lanes
+    int *refused;   // items 16 lanes could not plan, for a round of 32 lanes
     int *refused_count;
-    const int *wide;  // builds: this round takes these nwide items (once refused) instead of fresh ones
-    int nwide;
+    const int *wide;  // this round takes nwide of these (once refused): > 0 (builds) instead of fresh
+    int nwide;        // items, < 0 (a step's last round) all of them before fresh items
     int *pending;   // moves only: moves not done after the last round
     int div;        // builds: operations up to the points inserted or up to `few`, and 1 / div of
                     // them beyond (0: no such limit)
@@ -80,17 +80,26 @@ struct Rounds {
     int ops;        // room for operations of one round
 };
 
-// the round's operations: losers, then the wide list or fresh items (total: length of the queue)
-__device__ __forceinline__ void round_window(const Rounds &R, int b, int total, int &nlost, int &head, int &count)
+// items of the refused list that a round with nwide < 0 takes after its nlost losers
+__device__ __forceinline__ int round_all_refused(const Rounds &R, int nlost)
+{
+    return min(__ldcg(R.refused_count), max(0, R.ops - nlost));
+}
+
+// the round's operations: losers, nw items of the wide list, fresh items from `head` (total:
+// length of the queue)
+__device__ __forceinline__ void round_window(const Rounds &R, int b, int total, int &nlost, int &nw, int &head,
+                                             int &count)
 {
     nlost = __ldcg(R.lostcnt + b);
     head = __ldcg(R.head + b);
+    nw = R.nwide >= 0 ? R.nwide : round_all_refused(R, nlost);
     int lim = R.ops;
     if (R.div > 0) {
         const int in = R.base + head - nlost;
         lim = min(lim, max(max(64, in / R.div), min(in, R.few)));
     }
-    count = nlost + (R.nwide > 0 ? R.nwide : max(0, min(lim - nlost, total - head)));
+    count = nlost + nw + (R.nwide > 0 ? 0 : max(0, min(lim - nlost - nw, total - head)));
 }
 
 // priority of operation x of round b: the round first, then a different order of the
@@ -147,8 +156,9 @@ __device__ __forceinline__ int near_start(const Dev &d, const int *order, int n,
 
 // RL lanes per operation.  With fewer operations than warps every operation has a warp to
 // itself, so no warp is as long as the union of two operations' paths.  An operation
-// outside RL's limits goes to the list of the warp-wide path when `last` is set; otherwise a
-// move is planned again in the next round and an insertion goes to the refused list.
+// outside RL's limits goes to the list of the warp-wide path when `last` is set, otherwise to
+// the refused list: the triangulation changes little from round to round, so the same lanes
+// would refuse it again.  A move whose walk is too long goes to the warp-wide path at once.
 //
 // round_plan: `tid` of `nthreads` threads (whole warps), shared: one RegionShared per group of
 // the block.
@@ -158,11 +168,11 @@ __device__ __forceinline__ void round_plan(const Dev &d, const Rounds &R, int b,
                                            int nthreads)
 {
     constexpr bool MOVE = MODE != REGION_INSERT;
-    int nlost, head, count;
-    round_window(R, b, total, nlost, head, count);
+    int nlost, nw, head, count;  // (nw > 0 in rounds of 32 lanes only)
+    round_window(R, b, total, nlost, nw, head, count);
     const int off = __ldcg(R.off + b);
     if (tid == 0) {
-        R.head[b + 1] = R.nwide > 0 ? head : head + count - nlost;
+        R.head[b + 1] = head + count - nlost - nw;
         R.off[b + 1] = off + count;
     }
     constexpr int PER_WARP = 32 / RL;
@@ -175,9 +185,15 @@ __device__ __forceinline__ void round_plan(const Dev &d, const Rounds &R, int b,
     unsigned ex = 0, ti = 0, steps = 0;
     const int groups = alone ? warps : warps * PER_WARP;
     for (int x = alone ? tid / 32 : tid / RL; x < count; x += groups) {
-        const int item = x < nlost ? __ldcg(R.lost[b & 1] + x)
-                                   : (MOVE ? head + x - nlost
-                                           : __ldcg((R.nwide > 0 ? R.wide : B.queue + head) + x - nlost));
+        int item;
+        if (x < nlost) {
+            item = __ldcg(R.lost[b & 1] + x);
+        } else if (RL == 32 && x < nlost + nw) {
+            item = __ldcg(R.wide + x - nlost);
+        } else {
+            item = head + x - nlost - (RL == 32 ? nw : 0);
+            if (!MOVE) item = __ldcg(B.queue + item);
+        }
         RegionOut o;
         int4 *rec = R.rec + (size_t)x * (2 * RT);
         int rc, p;
@@ -207,7 +223,7 @@ __device__ __forceinline__ void round_plan(const Dev &d, const Rounds &R, int b,
         }
         ex += o.ex;
         ti += o.ti;
-        int nt = rc == RG_OK ? o.nt : (last || !MOVE ? -1 : 0);
+        int nt = rc == RG_OK ? o.nt : -1;
         if (rc == RG_VERTEX) {
             // q lies on a point: one that moves in this step may have left by the next round
             if (!MOVE) atomicCAS(d.status, 0, DEV_DUPLICATE);
@@ -222,7 +238,7 @@ __device__ __forceinline__ void round_plan(const Dev &d, const Rounds &R, int b,
         if (l == 0) {
             steps += o.steps;
             if (nt < 0) {
-                if (MOVE || last) R.left[atomicAdd(R.left_count, 1)] = item;
+                if (last || (MOVE && rc != RG_BAIL)) R.left[atomicAdd(R.left_count, 1)] = item;
                 else R.refused[atomicAdd(R.refused_count, 1)] = item;
             }
             R.hdr[x] = make_int4(item, nt, pr, o.k | o.ncav << 8 | o.edge << 24 | o.ghost << 25 | o.prop << 26);
@@ -260,8 +276,8 @@ template <bool MOVE>
 __device__ __forceinline__ void round_commit(const Dev &d, const Rounds &R, int b, const RoundMoves &M, int total,
                                              int *sum, int tid, int nthreads)
 {
-    int nlost, head, count;
-    round_window(R, b, total, nlost, head, count);
+    int nlost, nw, head, count;
+    round_window(R, b, total, nlost, nw, head, count);
     const int lane = threadIdx.x & (ROUND_LANES - 1);
     const unsigned gm = 0xffu << (threadIdx.x & 24);  // this operation's lanes
     int nwin = 0, nlose = 0, degs = 0, flips = 0, edges = 0, ghosts = 0, props = 0, hits = 0;
@@ -352,8 +368,8 @@ __global__ void __launch_bounds__(256) k_round_commit(Dev d, Rounds R, int b, Ro
 }
 
 // After the last of `rounds` rounds of a step: the owner words of every operation's
-// slots zero, and the moves not done (left out, losers of the last round, fresh items never
-// taken) to the kinetic kernel: few of them as a list, more on the lists of their
+// slots zero, and the moves not done (left out, losers of the last round, refused and fresh ones
+// never taken) to the kinetic kernel: few of them as a list, more on the lists of their
 // partitions, whose moves run one after another, so that moves that meet do not compete
 // (all 3,000 points of one partition moving at once filled the list of moves left for
 // later when every warp took one; 85,000 partitions' empty lists cost 100 us to look at).
@@ -370,11 +386,13 @@ __device__ __forceinline__ void round_clear(const Dev &d, const Rounds &R, int r
         if (s.w >= 0) d.tn[s.w].w = 0;
     }
     const int nleft = __ldcg(R.left_count), nlost = __ldcg(R.lostcnt + rounds), fresh = __ldcg(R.head + rounds);
-    const int pending = nleft + nlost + m - fresh;
+    const int ref0 = round_all_refused(R, __ldcg(R.lostcnt + rounds - 1)), nref = __ldcg(R.refused_count) - ref0;
+    const int pending = nleft + nlost + nref + m - fresh;
     if (tid == 0) *R.pending = pending;
     for (int i = tid; i < pending; i += nthreads) {
-        const int item = i < nleft ? __ldcg(R.left + i)
-                                   : (i < nleft + nlost ? __ldcg(R.lost[rounds & 1] + i - nleft) : fresh + i - nleft - nlost);
+        const int j = i - nleft, k = j - nlost, f = k - nref;
+        const int item = j < 0 ? __ldcg(R.left + i)
+                               : (k < 0 ? __ldcg(R.lost[rounds & 1] + j) : (f < 0 ? __ldcg(R.refused + ref0 + k) : fresh + f));
         const int inst = I.ninst > 1 ? csr_find(I.pofs, I.ninst + 1, gmoves[item].x) : 0;
         if (pending <= I.few_left) R.left[i] = item;
         else next[item] = atomicExch(head + partition_of(I, inst, bits, old_xy[item]), item);

@@ -80,3 +80,56 @@ def test_steps_of_several_windows():
         assert t.verify() == 0
         assert np.array_equal(t.export_points(), xy)
     assert t.stats()["fallbacks"] == 0
+
+
+def test_refused_moves_are_planned_by_32_lanes_once():
+    """150 hubs of degree 20 move at once: beyond 16 lanes, which refuse a move once and not in
+    every round (two refusals each counted 300 retries)."""
+    k, nr, c = 20, 150, 100000
+    a = 2 * np.pi * (np.arange(k) + 0.3) / k
+    r = 20000.0 + 7 * (np.arange(k) % 5)
+    rim = np.rint(np.stack([r * np.cos(a), r * np.sin(a)], 1)).astype(np.int64)
+    i = np.arange(nr)
+    at = np.stack([i % 13, i // 13], 1) * c + c // 2
+    xy = np.ascontiguousarray((np.concatenate([[[0, 0]], rim])[None] + at[:, None]).reshape(-1, 2).astype(np.int32))
+    t = _tri(grid=8, domain_bits=21, rebuild_ratio=2.0)
+    t.build(xy)
+    hubs = (k + 1) * i
+    before = t.stats()
+    for s in (3, -5):
+        mv = np.stack([hubs, xy[hubs, 0] + s, xy[hubs, 1] + 2], 1).astype(np.int32)
+        xy[hubs] = mv[:, 1:]
+        t.step(mv)
+        assert_same(t.export_triangles(), xy, "hubs")
+    st = t.stats()
+    assert st["retries"] - before["retries"] < 100
+    assert st["deletes"] - before["deletes"] == 2 * nr and st["fallbacks"] == 0
+
+
+def test_long_walks_are_walked_once_in_the_rounds():
+    """Two rows of 9,000 points: a jump from one end to the other crosses more triangles than the
+    rounds walk (4,096).  They give up once: 4,097 steps a move more than the kinetic kernel
+    alone, whose walks restart at random places (12,291 where three rounds tried).  1,000
+    jumps each: the walks are shorter than 1e5 steps and scatter by 1e4, their means by 450,
+    so the line is 8 of these from either figure."""
+    n, m = 9000, 100
+    x = 200 * np.arange(n, dtype=np.int64)
+    xy = np.concatenate([np.stack([x, 1000 + (x // 200) % 7], 1), np.stack([x + 90, 1300 + (x // 200) % 5], 1)])
+    xy = np.ascontiguousarray(xy.astype(np.int32))
+    steps = []
+    for kw in (dict(), dict(kinetic_warps=m)):
+        p = xy.copy()
+        t = _tri(grid=4, domain_bits=21, **kw)
+        t.build(p)
+        ids = 40 + 9 * np.arange(m)
+        before = t.stats()["walk_steps"]
+        for s in range(10):
+            to = 200 * (n - 60 - 7 * np.arange(m)) + 45 if s % 2 == 0 else 200 * ids + 45
+            mv = np.stack([ids, to, np.full(m, 1150)], 1).astype(np.int32)
+            p[ids] = mv[:, 1:]
+            t.step(mv)
+            assert t.verify() == 0
+        assert np.array_equal(t.export_points(), p)
+        assert_same(t.export_triangles(), p, "jumps")
+        steps.append((t.stats()["walk_steps"] - before) / (10 * m))
+    assert steps[0] - steps[1] < 8000
