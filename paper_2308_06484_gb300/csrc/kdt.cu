@@ -2007,7 +2007,7 @@ int d_values_impl(kdt *h, int N, int64_t *dist2, int64_t *cell_min2, kdt_dinfo *
     unsigned long long *sc = (unsigned long long *)h->dc_scal.p;  // [0] minimum, [1] largest degree
     unsigned long long init[2] = {(unsigned long long)INT64_MAX, 0ull};
     CK(cudaMemcpyAsync(sc, init, sizeof init, cudaMemcpyHostToDevice, st));
-    auto nth = N <= 2 ? k_nth_nn<2> : (N <= 4 ? k_nth_nn<4> : (N <= 8 ? k_nth_nn<8> : k_nth_nn<DC_MAX_N>));
+    auto nth = N <= 2 ? k_nth_nn<2> : (N <= 4 ? k_nth_nn<4> : (N <= 8 ? k_nth_nn<8> : (N <= 12 ? k_nth_nn<12> : k_nth_nn<DC_MAX_N>)));
     nth<<<(n + 127) / 128, 128, 0, st>>>(h->xy, h->pt_tri, TriHalf{h->tri}, TriHalf{h->tri + 1},
                                          h->order_valid ? (const int *)h->bord.p : nullptr, n, N, make_inst(h),
                                          h->cfg.domain_bits, dd, cm, sc, (int *)(sc + 1));
