@@ -1619,7 +1619,7 @@ int export_range(kdt *h, int s0, int nslots, int idbase, int np, int32_t *out, i
     h->stats.kernel_launches += 2;
     int32_t *dst = dev_out ? out : (int32_t *)h->exp_out.p;
     if (cap > 0) {
-        const size_t smem = ((2 + 2 * (size_t)EXB_ROWS) << s) * sizeof(int);
+        const size_t smem = exb_rows(s) * sizeof(unsigned long long) + (sizeof(int) * 2 << s);
         unsigned long long *rows = (unsigned long long *)h->exp_rows.p;
         k_exb_append<<<thread_grid(h, nslots, 256), 256, 0, st>>>(tv, nslots, cnt, rows, idbase, s, bits, total, most, cap);
         k_exb_sort<<<nb, EXB_THREADS, smem, st>>>(rows, off, s, bits, dst, total, most, cap);
@@ -1630,7 +1630,7 @@ int export_range(kdt *h, int s0, int nslots, int idbase, int np, int32_t *out, i
     *n_tri = h->hscal[S_TOTAL];
     if (*n_tri > cap) return KDT_ERR_CAPACITY;
     if (*n_tri == 0) return KDT_OK;
-    if (h->hscal[S_MOST] > EXB_ROWS << s) return export_placed(h, s0, nslots, idbase, np, out, cap, n_tri);
+    if (h->hscal[S_MOST] > exb_rows(s)) return export_placed(h, s0, nslots, idbase, np, out, cap, n_tri);
     if (!dev_out) {
         CK(cudaMemcpyAsync(out, dst, (size_t)*n_tri * sizeof(int3), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
@@ -1841,7 +1841,7 @@ int kdt_create(kdt **out, const kdt_config *cfg, int device, void *cuda_stream)
         cudaFuncSetAttribute(k_mlp_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TCS_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_mlp_grad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TG_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_exb_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(((2 + 2 * EXB_ROWS) << EXB_SHIFT) * sizeof(int))) != cudaSuccess) {
+                             (int)(exb_rows(EXB_SHIFT) * sizeof(unsigned long long) + (sizeof(int) * 2 << EXB_SHIFT))) != cudaSuccess) {
         kdt_destroy(h);
         return KDT_ERR_CUDA;
     }

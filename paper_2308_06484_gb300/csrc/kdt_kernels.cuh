@@ -1208,10 +1208,16 @@ __global__ void k_exp_sortseg(int n, const int *off, const int *cnt, int3 *out)
 // 1.45), 1.67 ms in buckets; 512 instances, 21.7e6 points: 3.24 -> 2.04; 1e6 points: 215 ->
 // 155 us; 1,000 points: 80 -> 46 us (four launches and one wait instead of eight and two).
 constexpr int EXB_ROWS = 7;     // rows a bucket may hold per first id (mean 2, up to 6 at the lowest ids)
+constexpr int EXB_MIN = 1536;   // ... and at least this many: one point of degree 40 among the lowest ids
+                                // fills 16 ids' 112 rows (100 rings of 40 points with their
+                                // centres: 196 us, with the second list placed, against 156)
 constexpr int EXB_SHIFT = 9;    // largest s: 33 KB a block
 constexpr int EXB_THREADS = 256;
 constexpr int EXB_PAD = 8;      // ints between two buckets' counters: a sector each, or the atomics of many
                                 // buckets queue at one
+
+// rows a bucket of 2^s ids may hold
+__host__ __device__ constexpr int exb_rows(int s) { return EXB_ROWS << s > EXB_MIN ? EXB_ROWS << s : EXB_MIN; }
 
 // rows per bucket
 __global__ void k_exb_count(TriHalf tv, int nslots, int *cnt, int idbase, int s)
@@ -1275,7 +1281,7 @@ __global__ void __launch_bounds__(1024) k_exb_scan(int *cnt, int nb, int *off, i
 __global__ void k_exb_append(TriHalf tv, int nslots, int *cur, unsigned long long *rows, int idbase, int s, int bits,
                              const int *total, const int *most, long long cap)
 {
-    if (__ldcg(total) > cap || __ldcg(most) > EXB_ROWS << s) return;
+    if (__ldcg(total) > cap || __ldcg(most) > exb_rows(s)) return;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nslots; t += gridDim.x * blockDim.x) {
         const int4 v = __ldcg(tv + t);
         if (!finite_alive(v)) continue;
@@ -1303,11 +1309,11 @@ __global__ void __launch_bounds__(EXB_THREADS) k_exb_sort(const unsigned long lo
                                                           int bits, int *out, const int *total, const int *most,
                                                           long long cap)
 {
-    if (__ldcg(total) > cap || __ldcg(most) > EXB_ROWS << s) return;
+    if (__ldcg(total) > cap || __ldcg(most) > exb_rows(s)) return;
     extern __shared__ unsigned long long exb[];
     const int ids = 1 << s, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned long long *r = exb;
-    int *start = reinterpret_cast<int *>(exb + (EXB_ROWS << s)), *fill = start + ids;
+    int *start = reinterpret_cast<int *>(exb + exb_rows(s)), *fill = start + ids;
     __shared__ int ws[EXB_THREADS / 32];
     const int base = off[blockIdx.x], n = off[blockIdx.x + 1] - base;
     for (int i = threadIdx.x; i < ids; i += EXB_THREADS) fill[i] = 0;
