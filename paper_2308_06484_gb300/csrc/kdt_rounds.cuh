@@ -409,10 +409,14 @@ __global__ void k_round_clear(Dev d, Rounds R, int rounds, int m, Inst I, int bi
 
 // A whole small step in one block: clearing, intake, rounds until every move is done (or a
 // round does none), and what is left to the kinetic kernel.  The kernels it replaces take
-// 2 to 4 us each whatever they do, and a step of a few moves is three rounds of them: 1,000
-// points, 13 moves, 67 -> 61 us a step with a wait after each, 500 -> 450 us for eight and an
-// export.
-constexpr int SMALL_MOVES = 64;      // two moves a warp, one after the other
+// 2 to 4 us each whatever they do, and a step of a few moves is three rounds of them; but one
+// block plans 16 moves at a time and the whole GPU all of them.  us a step with a wait after
+// each, one block / whole GPU:
+//   moves                                     4      16      32      40      48      64
+//   1e6 points, short moves               39 / 48  38 / 51  47 / 51  54 / 54  51 / 51  63 / 51
+//   1,000 points, one unit                38 / 49  51 / 62  56 / 61  67 / 65  74 / 71  97 / 99
+//   2e5 points, jumps of two spacings     39 / 52  42 / 53  54 / 56  63 / 57  69 / 59  84 / 65
+constexpr int SMALL_MOVES = 32;      // two moves a warp, one after the other
 constexpr int SMALL_THREADS = 512;
 constexpr int SMALL_ROUNDS = 16;
 constexpr int SMALL_CELLS = 8192;    // partitions one block clears in passing

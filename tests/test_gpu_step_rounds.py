@@ -133,3 +133,18 @@ def test_long_walks_are_walked_once_in_the_rounds():
         assert_same(t.export_triangles(), p, "jumps")
         steps.append((t.stats()["walk_steps"] - before) / (10 * m))
     assert steps[0] - steps[1] < 8000
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+def test_small_steps_end_at_32_moves(graph):
+    """Up to two moves a warp of one block take its three launches, more the whole GPU's."""
+    n = 5000
+    xy = W.uniform_points(n, 24, 8)
+    t = _tri(grid=4, domain_bits=24, use_graph=graph)
+    t.build(xy)
+    rng = np.random.default_rng(3)
+    for i, m in enumerate((1, 31, 32, 33, 64, 65, 32, 16, 17)):
+        before = t.stats()["kernel_launches"]
+        t.step(_shift(xy, rng.permutation(n)[:m], 50 + i))
+        assert (t.stats()["kernel_launches"] - before == 3) == (m <= 32)
+        assert_same(t.export_triangles(), xy, "%d moves" % m)
