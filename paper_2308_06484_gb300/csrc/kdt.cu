@@ -389,19 +389,21 @@ int kinetic_blocks(kdt *h)
 
 // Certify slots [s0, s0 + nslots) (or the dirty list when !full), then repair until
 // no violation is left.  A full pass must see `wraps` hull windings (one per
-// instance in the range).  Returns a CUDA/ABI error; the device status goes to
+// instance in the range) and, when the range is `whole` (not during a build), a triangle
+// in every slot.  Returns a CUDA/ABI error; the device status goes to
 // *dev_status.
-int certify_and_repair(kdt *h, bool full, int s0, int nslots, int wraps, int *dev_status)
+int certify_and_repair(kdt *h, bool full, int s0, int nslots, int wraps, int *dev_status, bool whole = true)
 {
     Dev d = make_dev(h);
     if (full && d.retry_cap < 4096) d.retry_cap = 4096;
     int lo = 0;
     for (int round = 0; round < 64; ++round) {
-        CK(cudaMemsetAsync(h->scal + S_VIOL, 0, sizeof(int), h->stream));
+        CK(cudaMemsetAsync(h->scal + S_VIOL, 0, 2 * sizeof(int), h->stream));  // and S_DEAD
         CK(cudaMemsetAsync(h->scal + S_WRAPS, 0, sizeof(int), h->stream));
         if (full) {
             k_certify_all<<<thread_grid(h, nslots, 256), 256, 0, h->stream>>>(d, s0, nslots, h->viol, h->scal + S_VIOL,
-                                                                             h->viol_cap, h->scal + S_WRAPS);
+                                                                             h->viol_cap, h->scal + S_WRAPS,
+                                                                             whole ? h->scal + S_DEAD : nullptr);
         } else {
             k_certify<<<thread_grid(h, 65536, 256), 256, 0, h->stream>>>(d, lo, h->viol, h->scal + S_VIOL,
                                                                         h->viol_cap);
@@ -415,7 +417,7 @@ int certify_and_repair(kdt *h, bool full, int s0, int nslots, int wraps, int *de
         h->stats.violations += nv;
         if (nv == 0) {
             // every edge is locally Delaunay; after a full pass each hull winds once
-            if (full && h->hscal[S_WRAPS] != wraps) *dev_status = DEV_INTERNAL;
+            if (full && (h->hscal[S_WRAPS] != wraps || h->hscal[S_DEAD] != 0)) *dev_status = DEV_INTERNAL;
             return 0;
         }
         if (nv > h->viol_cap) nv = h->viol_cap;  // the rest is found again next round
@@ -593,7 +595,7 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
             h->stats.kernel_launches++;
             CK(cudaGetLastError());
             int ds = 0;  // (the rounds' plans need every edge locally Delaunay)
-            if (certify_and_repair(h, true, s0, nslots, ni, &ds)) return KDT_ERR_CUDA;
+            if (certify_and_repair(h, true, s0, nslots, ni, &ds, false)) return KDT_ERR_CUDA;
             if (ds) return dev_to_abi(ds);
             left_done = nleft;
         }
@@ -689,7 +691,7 @@ int rebuild_instance(kdt *h, int i)
     h->stats.kernel_launches += 2;
     if (sync_scalars(h)) return KDT_ERR_CUDA;
     if (h->hscal[S_THIRD] == INT_MAX) return KDT_ERR_DEGENERATE;
-    k_init<<<1, 1, 0, st>>>(d, order, h->scal + S_THIRD, h->scal + S_TRIS, s0);
+    k_init<<<1, 1, 0, st>>>(d, order, h->scal + S_THIRD, s0);
     h->stats.kernel_launches++;
     int K = 0;
     while ((1ll << (K + 1)) < (long long)n) ++K;
@@ -718,11 +720,11 @@ int rebuild_batch(kdt *h)
     Dev d = make_dev(h);
     d.dirty_cap = 0;
     if (d.retry_cap < 32768) d.retry_cap = 32768;
-    // per-instance tables: bbox (4), hk, hshift, hbase (ni + 1), third, tri_count
-    const size_t tab_ints = 4 * (size_t)ni + 5 * (size_t)ni + 1;
+    // per-instance tables: bbox (4), hk, hshift, hbase (ni + 1), third
+    const size_t tab_ints = 4 * (size_t)ni + 4 * (size_t)ni + 1;
     if (grow(h->btab, tab_ints * sizeof(int))) return KDT_ERR_CUDA;
-    int *bbox = (int *)h->btab.p, *hk = bbox + 4 * ni, *hsh = hk + ni, *third = hsh + ni, *tcount = third + ni;
-    unsigned *hbase = (unsigned *)(tcount + ni);
+    int *bbox = (int *)h->btab.p, *hk = bbox + 4 * ni, *hsh = hk + ni, *third = hsh + ni;
+    unsigned *hbase = (unsigned *)(third + ni);
     std::vector<int> hb(4 * (size_t)ni);
     for (int i = 0; i < ni; ++i) {
         hb[4 * i] = INT_MAX;
@@ -782,7 +784,7 @@ int rebuild_batch(kdt *h)
     CK(cudaStreamSynchronize(st));
     for (int i = 0; i < ni; ++i)
         if (th[i] == INT_MAX) return KDT_ERR_DEGENERATE;
-    k_init_batch<<<thread_grid(h, ni, 128), 128, 0, st>>>(d, order, third, h->d_pofs, h->d_tofs, ni, tcount);
+    k_init_batch<<<thread_grid(h, ni, 128), 128, 0, st>>>(d, order, third, h->d_pofs, h->d_tofs, ni);
     h->stats.kernel_launches++;
     // the items of every level: instance i's positions (2j+1) * 2^level below n_i
     std::vector<int> lv((size_t)(Kmax + 1) * (ni + 1), 0);

@@ -20,7 +20,7 @@ constexpr int DEV_FAR = 11;     // a move went farther than the rebuild rule all
 
 // small device block of scalars
 enum Slot : int {
-    S_STATUS = 0, S_DIRTY = 1, S_VIOL = 2, S_TRIS = 3, S_DEFER = 4, S_THIRD = 5,
+    S_STATUS = 0, S_DIRTY = 1, S_VIOL = 2, S_DEAD = 3, S_DEFER = 4, S_THIRD = 5,
     S_MINX = 6, S_MINY = 7, S_MAXX = 8, S_MAXY = 9, S_TOTAL = 10, S_BAD = 11, S_ALIVE = 12,
     S_WRAPS = 13, S_FAILPT = 14, S_DONE = 15, S_CERTPEND = 16, S_TICKET = 17, S_DNEXT = 18,
     S_DRUN = 19,  // warps running a move taken from the deferred list (kinetic launch)
@@ -891,8 +891,10 @@ __global__ void k_certify(Dev d, int lo, int *viol, int *viol_count, int viol_ca
         certify_one(d, d.dirty[i], viol, viol_count, viol_cap, &ex, &ti);
 }
 
-// certify every slot (after a build, or when the dirty list overflowed)
-__global__ void k_certify_all(Dev d, int s0, int nslots, int *viol, int *viol_count, int viol_cap, int *wraps)
+// certify every slot (after a build, or when the dirty list overflowed); dead (null while a
+// build goes on): slots without a triangle, of which a triangulation has none
+__global__ void k_certify_all(Dev d, int s0, int nslots, int *viol, int *viol_count, int viol_cap, int *wraps,
+                              int *dead)
 {
     unsigned ex = 0, ti = 0;
     for (int t = s0 + blockIdx.x * blockDim.x + threadIdx.x; t < s0 + nslots; t += gridDim.x * blockDim.x) {
@@ -901,6 +903,8 @@ __global__ void k_certify_all(Dev d, int s0, int nslots, int *viol, int *viol_co
         if ((v.w & ALIVE) && (v.x < 0 || v.y < 0 || v.z < 0)) {
             int wr = hull_wrap(d, v, __ldcg(d.tn + t));
             if (wr) atomicAdd(wraps, wr);
+        } else if (dead && !(v.w & ALIVE)) {
+            atomicAdd(dead, 1);
         }
     }
 }
@@ -1006,7 +1010,7 @@ __global__ void k_third(const int2 *xy, int n, const int *order, int *third)
 }
 
 // The first triangle (a, b, c) and its three ghosts (c,b,inf), (a,c,inf), (b,a,inf).
-__global__ void k_init(Dev d, const int *order, const int *third, int *tri_count, int s0)
+__global__ void k_init(Dev d, const int *order, const int *third, int s0)
 {
     int a = order[0], b = order[1], c = order[*third];
     if (orient2d(d.xy[a], d.xy[b], d.xy[c]) < 0) {
@@ -1027,7 +1031,6 @@ __global__ void k_init(Dev d, const int *order, const int *third, int *tri_count
     d.pt_tri[a] = t0;
     d.pt_tri[b] = t0;
     d.pt_tri[c] = t0;
-    *tri_count = s0 + 4;
 }
 
 // ------------------------------------------------------------------ batched build
@@ -1117,8 +1120,7 @@ __global__ void k_third_batch(const int2 *xy, int n, const int *order, const int
 }
 
 // per instance: its first triangle and three ghosts at its first slots (as k_init)
-__global__ void k_init_batch(Dev d, const int *order, const int *third, const int *pofs, const int *tofs, int ninst,
-                             int *tri_count)
+__global__ void k_init_batch(Dev d, const int *order, const int *third, const int *pofs, const int *tofs, int ninst)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ninst; i += gridDim.x * blockDim.x) {
         const int p0 = pofs[i], s0 = tofs[i];
@@ -1141,7 +1143,6 @@ __global__ void k_init_batch(Dev d, const int *order, const int *third, const in
         d.pt_tri[a] = t0;
         d.pt_tri[b] = t0;
         d.pt_tri[c] = t0;
-        tri_count[i] = s0 + 4;
     }
 }
 
