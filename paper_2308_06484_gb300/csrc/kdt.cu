@@ -61,7 +61,8 @@ constexpr int SMALL_GRAPH = STEP_CLASSES, STEP_GRAPHS = STEP_CLASSES + 1;
 
 constexpr long long class_moves(int c)
 {
-    return c < STEP_MANY_CLASS ? std::min(2048ll << 2 * c, STEP_MANY - 1ll) : (long long)ROUND_OPS << (c - STEP_MANY_CLASS);
+    return c < STEP_MANY_CLASS ? std::min(2048ll << 2 * c, STEP_MANY - 1ll)
+                               : (long long)ROUND_OPS << (c - STEP_MANY_CLASS);
 }
 
 int step_class(long long m)
@@ -557,9 +558,14 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
     long long total = 0;
     for (int l = 0; l < levels; ++l) total += lv[(size_t)l * (ni + 1) + ni];
     const long long np = total + ni;
-    const int ops = (int)std::min<long long>(ROUND_OPS, std::max<long long>(64, std::max<long long>(np / BUILD_DIV, std::min<long long>(np, BUILD_FEW)) + 64));
-    if (grow(h->rb_cnt, round_counter_ints(ROUND_MAX) * sizeof(int)) || grow(h->rb_lost, 2 * (size_t)ops * sizeof(int)) ||
-        grow(h->rb_hdr, (size_t)ops * sizeof(int4)) || grow(h->rb_rec, (size_t)ops * 2 * RT * sizeof(int4)) ||
+    // operations of a round with `in` points in
+    auto window = [](long long in) {
+        return std::max<long long>({64ll, in / BUILD_DIV, std::min<long long>(in, BUILD_FEW)});
+    };
+    const int ops = (int)std::min<long long>(ROUND_OPS, window(np) + 64);
+    if (grow(h->rb_cnt, round_counter_ints(ROUND_MAX) * sizeof(int)) ||
+        grow(h->rb_lost, 2 * (size_t)ops * sizeof(int)) || grow(h->rb_hdr, (size_t)ops * sizeof(int4)) ||
+        grow(h->rb_rec, (size_t)ops * 2 * RT * sizeof(int4)) ||
         grow(h->rb_queue, (size_t)np * sizeof(int)) || grow(h->rb_left, (size_t)np * sizeof(int)) ||
         grow(h->rb_ref, (size_t)np * sizeof(int)))
         return KDT_ERR_CUDA;
@@ -578,7 +584,8 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
         if (items <= 0) continue;
         long long stride = std::max(1ll, std::llround(0.6180339887498949 * (double)items));
         while (std::gcd(stride, (long long)items) != 1) ++stride;
-        k_build_queue<<<thread_grid(h, items, 256), 256, 0, st>>>(B, ni > 1 ? dlv + (size_t)l * (ni + 1) : h->d_pofs, l, items, (int)stride,
+        const int *lvoff = ni > 1 ? dlv + (size_t)l * (ni + 1) : h->d_pofs;
+        k_build_queue<<<thread_grid(h, items, 256), 256, 0, st>>>(B, lvoff, l, items, (int)stride,
                                                                  (int *)h->rb_queue.p + at);
         h->stats.kernel_launches++;
         at += items;
@@ -611,8 +618,7 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
         }
         // rounds until the points in have grown fourfold, if every operation won
         for (long long est = in; b < ROUND_MAX && (k < BUILD_ROUNDS || (est < 4 * in && est < np)); ++b, ++k) {
-            const long long most = std::min<long long>(
-                {(long long)ops, (long long)pend, std::max<long long>({64ll, est / BUILD_DIV, std::min<long long>(est, BUILD_FEW)})});
+            const long long most = std::min<long long>({(long long)ops, (long long)pend, window(est)});
             const bool wide = 32 * most <= (long long)ROUND_THREADS * 32 * sm_count(h->device);
             launch_round<REGION_INSERT>(h, st, d, R, b, most, M, B, wide, wide);
             est = std::min(est + most, np);
@@ -633,9 +639,10 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
     k_clear_owner<<<thread_grid(h, nslots, 256), 256, 0, st>>>(d.tn, s0, nslots);
     h->stats.kernel_launches++;
     if (pend > 0 || nref > ref_done) {  // (ROUND_MAX rounds)
-        k_build_rest<<<thread_grid(h, pend + nref - ref_done, 256), 256, 0, st>>>(R, b, B, R.refused + ref_done, nref - ref_done);
+        const int rest = pend + nref - ref_done;
+        k_build_rest<<<thread_grid(h, rest, 256), 256, 0, st>>>(R, b, B, R.refused + ref_done, nref - ref_done);
         h->stats.kernel_launches++;
-        nleft += pend + nref - ref_done;
+        nleft += rest;
     }
     if (nleft > left_done)
         launch_insert_warps(h, d, R.left + left_done, nleft - left_done, left_warps(in), B, 0, nullptr);
@@ -665,8 +672,8 @@ int rebuild_instance(kdt *h, int i)
     CK(cudaMemcpyAsync(h->scal + S_THIRD, &third0, sizeof(int), cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(h->tri + 2 * (size_t)s0, 0, 2 * (size_t)capi * sizeof(int4), st));
     k_fill_int<<<thread_grid(h, n, 256), 256, 0, st>>>(h->pt_tri + p0, n, -1);
-    k_range<<<std::min(thread_grid(h, n, 256), 4 * sm_count(h->device)), 256, 0, st>>>(h->xy + p0, n, h->cfg.domain_bits, h->scal + S_STATUS,
-                                                    h->scal + S_MINX);
+    k_range<<<std::min(thread_grid(h, n, 256), 4 * sm_count(h->device)), 256, 0, st>>>(
+        h->xy + p0, n, h->cfg.domain_bits, h->scal + S_STATUS, h->scal + S_MINX);
     h->stats.kernel_launches += 2;
     if (sync_scalars(h)) return KDT_ERR_CUDA;
     if (h->hscal[S_STATUS]) return dev_to_abi(h->hscal[S_STATUS]);
@@ -991,8 +998,9 @@ void free_state(kdt *h)
     h->pfeat = nullptr;
     h->ppart = nullptr;
     h->mcap = 0; h->dirty_cap = 0; h->scan_tmp_cap = 0; h->rm_cap = 0;
-    Buf *bs[] = {&h->key, &h->bord, &h->hist, &h->hoff, &h->exp_cnt, &h->exp_off, &h->exp_fill, &h->exp_out, &h->exp_rows,
-                 &h->btab, &h->blev, &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left, &h->rb_ref,
+    Buf *bs[] = {&h->key, &h->bord, &h->hist, &h->hoff, &h->exp_cnt, &h->exp_off, &h->exp_fill, &h->exp_out,
+                 &h->exp_rows, &h->btab, &h->blev,
+                 &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left, &h->rb_ref,
                  &h->rm_cnt, &h->rm_lost, &h->rm_hdr, &h->rm_rec, &h->rm_slots, &h->rm_left, &h->rm_ref,
                  &h->dc_dist, &h->dc_cmin, &h->dc_scal};
     for (Buf *b : bs) free_buf(*b);
@@ -1202,7 +1210,8 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
 {
     const bool rounds = step_in_rounds(h), small = which == SMALL_GRAPH;
     const int nrounds = small ? SMALL_ROUNDS : class_rounds(which);
-    const int cap = !from_ctl ? mi : (rounds && !small ? (int)std::min<long long>(h->mcap, class_moves(which)) : h->mcap);
+    int cap = mi;
+    if (from_ctl) cap = rounds && !small ? (int)std::min<long long>(h->mcap, class_moves(which)) : h->mcap;
     Inst I = make_inst(h);
     // the step's control words and move offsets, from pinned host memory (a captured
     // copy reads them when the graph runs)
@@ -1223,9 +1232,10 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
         if (h->cfg.timing) CK(cudaEventRecordWithFlags(h->ev0, st, evflags0));
         // (a small step's moves push a few entries each onto the deferred list)
         const int ndef = std::min(h->mcap, 8 * SMALL_MOVES);
-        k_step_small<<<1, SMALL_THREADS, 0, st>>>(d, mp, mi, I, h->cfg.domain_bits, h->scal, S_NUM, h->head, h->ncells_cap,
-                                                  h->next, h->deferred, ndef, h->old_xy, h->gmoves, h->dloc2, far2(h), R,
-                                                  (int *)h->rm_cnt.p, (int)round_counter_ints(h->rm_layout));
+        k_step_small<<<1, SMALL_THREADS, 0, st>>>(d, mp, mi, I, h->cfg.domain_bits, h->scal, S_NUM, h->head,
+                                                  h->ncells_cap, h->next, h->deferred, ndef, h->old_xy, h->gmoves,
+                                                  h->dloc2, far2(h), R, (int *)h->rm_cnt.p,
+                                                  (int)round_counter_ints(h->rm_layout));
         return enqueue_kinetic(h, st, d, I, from_ctl, ndef);
     }
     // scalars zero, partition lists empty, deferred entries -1: one kernel
@@ -1265,10 +1275,9 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
                                                              net ? h->pguess : nullptr, ordered ? h->pcost : nullptr,
                                                              tensor ? h->pfeat : nullptr, tensor ? h->ppart : nullptr);
         if (tensor)
-            k_mlp_tc<1><<<tc_grid(h, cap), TC_THREADS, TCS_BYTES, st>>>(h->mlp_w, h->pfeat, mi, from_ctl ? h->ctl : nullptr,
-                                                                  nullptr, h->ppart, h->gmoves, h->pguess,
-                                                                  ordered ? h->pcost : nullptr,
-                                                                  h->counters + C_TC_FAIL);
+            k_mlp_tc<1><<<tc_grid(h, cap), TC_THREADS, TCS_BYTES, st>>>(
+                h->mlp_w, h->pfeat, mi, from_ctl ? h->ctl : nullptr, nullptr, h->ppart, h->gmoves, h->pguess,
+                ordered ? h->pcost : nullptr, h->counters + C_TC_FAIL);
     }
     if (ordered) {
         const int ostride = h->qhist || h->cfg.partition_order ? 1 : h->stride;
@@ -1621,10 +1630,10 @@ int export_range(kdt *h, int s0, int nslots, int idbase, int np, int32_t *out, i
     h->stats.kernel_launches += 2;
     int32_t *dst = dev_out ? out : (int32_t *)h->exp_out.p;
     if (cap > 0) {
-        const size_t smem = exb_rows(s) * sizeof(unsigned long long) + (sizeof(int) * 2 << s);
         unsigned long long *rows = (unsigned long long *)h->exp_rows.p;
-        k_exb_append<<<thread_grid(h, nslots, 256), 256, 0, st>>>(tv, nslots, cnt, rows, idbase, s, bits, total, most, cap);
-        k_exb_sort<<<nb, EXB_THREADS, smem, st>>>(rows, off, s, bits, dst, total, most, cap);
+        k_exb_append<<<thread_grid(h, nslots, 256), 256, 0, st>>>(tv, nslots, cnt, rows, idbase, s, bits, total, most,
+                                                                 cap);
+        k_exb_sort<<<nb, EXB_THREADS, exb_shared(s), st>>>(rows, off, s, bits, dst, total, most, cap);
         h->stats.kernel_launches += 2;
     }
     CK(cudaGetLastError());
@@ -1654,8 +1663,8 @@ int build_quadtree(kdt *h)
     int init_bbox[4] = {INT_MAX, INT_MAX, INT_MIN, INT_MIN};
     CK(cudaMemsetAsync(h->scal, 0, S_NUM * sizeof(int), st));
     CK(cudaMemcpyAsync(h->scal + S_MINX, init_bbox, sizeof init_bbox, cudaMemcpyHostToDevice, st));
-    k_range<<<std::min(thread_grid(h, n, 256), 4 * sm_count(h->device)), 256, 0, st>>>(h->xy, n, h->cfg.domain_bits, h->scal + S_STATUS,
-                                                    h->scal + S_MINX);
+    k_range<<<std::min(thread_grid(h, n, 256), 4 * sm_count(h->device)), 256, 0, st>>>(
+        h->xy, n, h->cfg.domain_bits, h->scal + S_STATUS, h->scal + S_MINX);
     if (sync_scalars(h)) return KDT_ERR_CUDA;
     const int x0 = h->hscal[S_MINX], y0 = h->hscal[S_MINY];
     const long long ext = std::max((long long)h->hscal[S_MAXX] - x0, (long long)h->hscal[S_MAXY] - y0) + 1;
@@ -1843,7 +1852,7 @@ int kdt_create(kdt **out, const kdt_config *cfg, int device, void *cuda_stream)
         cudaFuncSetAttribute(k_mlp_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TCS_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_mlp_grad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TG_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_exb_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(exb_rows(EXB_SHIFT) * sizeof(unsigned long long) + (sizeof(int) * 2 << EXB_SHIFT))) != cudaSuccess) {
+                             (int)exb_shared(EXB_SHIFT)) != cudaSuccess) {
         kdt_destroy(h);
         return KDT_ERR_CUDA;
     }
@@ -2009,7 +2018,11 @@ int d_values_impl(kdt *h, int N, int64_t *dist2, int64_t *cell_min2, kdt_dinfo *
     unsigned long long *sc = (unsigned long long *)h->dc_scal.p;  // [0] minimum, [1] largest degree
     unsigned long long init[2] = {(unsigned long long)INT64_MAX, 0ull};
     CK(cudaMemcpyAsync(sc, init, sizeof init, cudaMemcpyHostToDevice, st));
-    auto nth = N <= 2 ? k_nth_nn<2> : (N <= 4 ? k_nth_nn<4> : (N <= 8 ? k_nth_nn<8> : (N <= 12 ? k_nth_nn<12> : k_nth_nn<DC_MAX_N>)));
+    auto nth = k_nth_nn<DC_MAX_N>;
+    if (N <= 2) nth = k_nth_nn<2>;
+    else if (N <= 4) nth = k_nth_nn<4>;
+    else if (N <= 8) nth = k_nth_nn<8>;
+    else if (N <= 12) nth = k_nth_nn<12>;
     nth<<<(n + 127) / 128, 128, 0, st>>>(h->xy, h->pt_tri, TriHalf{h->tri}, TriHalf{h->tri + 1},
                                          h->order_valid ? (const int *)h->bord.p : nullptr, n, N, make_inst(h),
                                          h->cfg.domain_bits, dd, cm, sc, (int *)(sc + 1));
@@ -2314,9 +2327,9 @@ int kdt_mlp_loss_grad_tc(kdt *h, const uint16_t *params_bf16, const float *x, co
     const int blocks = (int)std::min<long long>((rows + TC_M - 1) / TC_M, sm_count(h->device));
     if (int rc = ensure_mlp_part(h, blocks)) return rc;
     float *part_loss = h->mlp_part + (size_t)h->mlp_part_blocks * MLP_PARAMS;
-    k_mlp_grad_tc<<<blocks, TG_THREADS, TG_BYTES, h->stream>>>((const unsigned short *)params_bf16, x, (const int *)labels,
-                                                        (const long long *)index, rows, lam, h->mlp_part, part_loss,
-                                                        h->counters + C_TC_FAIL);
+    k_mlp_grad_tc<<<blocks, TG_THREADS, TG_BYTES, h->stream>>>(
+        (const unsigned short *)params_bf16, x, (const int *)labels, (const long long *)index, rows, lam, h->mlp_part,
+        part_loss, h->counters + C_TC_FAIL);
     k_mlp_reduce<<<REDUCE_BLOCKS, 32 * REDUCE_WARPS, 0, h->stream>>>(h->mlp_part, part_loss, blocks, rows, grad, loss);
     h->stats.kernel_launches += 2;
     CK(cudaGetLastError());

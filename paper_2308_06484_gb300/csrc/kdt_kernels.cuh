@@ -1219,6 +1219,8 @@ constexpr int EXB_PAD = 8;      // ints between two buckets' counters: a sector 
 
 // rows a bucket of 2^s ids may hold
 __host__ __device__ constexpr int exb_rows(int s) { return EXB_ROWS << s > EXB_MIN ? EXB_ROWS << s : EXB_MIN; }
+// shared memory of k_exb_sort: the rows, starts and cursors of the ids
+constexpr size_t exb_shared(int s) { return exb_rows(s) * sizeof(unsigned long long) + (2 * sizeof(int) << s); }
 
 // rows per bucket
 __global__ void k_exb_count(TriHalf tv, int nslots, int *cnt, int idbase, int s)
@@ -1323,7 +1325,8 @@ __global__ void __launch_bounds__(EXB_THREADS) k_exb_sort(const unsigned long lo
     for (int i = threadIdx.x; i < n; i += EXB_THREADS) atomicAdd(fill + (int)(__ldg(in + i) >> 2 * bits), 1);
     __syncthreads();
     // exclusive scan of the counts, `per` ids a thread
-    const int per = (ids + EXB_THREADS - 1) / EXB_THREADS, lo = min(ids, (int)threadIdx.x * per), hi = min(ids, lo + per);
+    const int per = (ids + EXB_THREADS - 1) / EXB_THREADS;
+    const int lo = min(ids, (int)threadIdx.x * per), hi = min(ids, lo + per);
     int sum = 0;
     for (int i = lo; i < hi; ++i) sum += fill[i];
     int x = sum;
@@ -1362,7 +1365,8 @@ __global__ void __launch_bounds__(EXB_THREADS) k_exb_sort(const unsigned long lo
     for (int i = threadIdx.x; i < 3 * n; i += EXB_THREADS) {
         const int j = i / 3, f = i - 3 * j;
         const unsigned long long w = r[j];
-        out[3ll * base + i] = f == 0 ? a0 + (int)(w >> 2 * bits) : (f == 1 ? (int)((w >> bits) & mask) : (int)(w & mask));
+        out[3ll * base + i] =
+            f == 0 ? a0 + (int)(w >> 2 * bits) : (f == 1 ? (int)((w >> bits) & mask) : (int)(w & mask));
     }
 }
 

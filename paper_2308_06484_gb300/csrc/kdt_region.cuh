@@ -60,7 +60,6 @@ struct RegionOut {
     int ncav;         // cavity size
     int edge, ghost;  // q lay on an edge / outside the hull
     int vtx;          // RG_VERTEX: the point q coincides with
-    int t0;           // a triangle of the store near q (the next attempt's start), or -1
     unsigned ex, ti;  // exact predicate calls, ties (this lane's)
     int steps;        // triangles walked through
     int prop;         // the learned proposal: 0 none, 1 a guess, 3 a guess whose triangle holds q
@@ -104,7 +103,6 @@ __device__ __forceinline__ int region_plan(const D &d, RegionShared<RL> &sh, int
     o.edge = 0;
     o.ghost = 0;
     o.vtx = -1;
-    o.t0 = -1;
     o.ex = 0;
     o.ti = 0;
     o.steps = 0;
@@ -349,14 +347,12 @@ __device__ __forceinline__ int region_plan(const D &d, RegionShared<RL> &sh, int
                     const int zeros = (o0 == 0) + (o1 == 0) + (o2 == 0);
                     if (zeros >= 2) {
                         o.vtx = o0 != 0 ? v.x : (o1 != 0 ? v.y : v.z);
-                        o.t0 = t;
                         return RG_VERTEX;
                     }
                     o.edge = zeros;
                 }
             }
             if (go < 0) {
-                o.t0 = t;
                 if (l == 0) {
                     sh.gs[0] = t;
                     sh.gv[0][0] = v.x;
@@ -374,7 +370,7 @@ __device__ __forceinline__ int region_plan(const D &d, RegionShared<RL> &sh, int
             }
             t = rcomp(n, go) >> 2;
         }
-        if (MOVE && votes(l < k && S == o.t0)) return RG_BAIL;  // (q is outside the star)
+        if (MOVE && votes(l < k && S == t)) return RG_BAIL;  // (q is outside the star)
     }
     // ---- 3. the cavity: the hole and ring triangles in conflict with q
     if (MOVE) {
@@ -390,7 +386,6 @@ __device__ __forceinline__ int region_plan(const D &d, RegionShared<RL> &sh, int
             out[2 * l] = make_int4(p, id, idn, 1);
             out[2 * l + 1] = make_int4(~O, (Sn << 2) | 2, (Sp << 2) | 1, S);
         }
-        o.t0 = sh1(S, 0);
         o.nt = k;
         o.ncav = k - 2;
         __syncwarp(gm);
@@ -571,7 +566,6 @@ __device__ __forceinline__ int region_plan(const D &d, RegionShared<RL> &sh, int
     }
     o.nt = nt;
     o.ncav = ncav;
-    if (o.t0 < 0) o.t0 = sh.pool[0];
     __syncwarp(gm);
     return RG_OK;
 }

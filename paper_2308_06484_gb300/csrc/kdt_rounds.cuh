@@ -391,8 +391,10 @@ __device__ __forceinline__ void round_clear(const Dev &d, const Rounds &R, int r
     if (tid == 0) *R.pending = pending;
     for (int i = tid; i < pending; i += nthreads) {
         const int j = i - nleft, k = j - nlost, f = k - nref;
-        const int item = j < 0 ? __ldcg(R.left + i)
-                               : (k < 0 ? __ldcg(R.lost[rounds & 1] + j) : (f < 0 ? __ldcg(R.refused + ref0 + k) : fresh + f));
+        int item = fresh + f;
+        if (j < 0) item = __ldcg(R.left + i);
+        else if (k < 0) item = __ldcg(R.lost[rounds & 1] + j);
+        else if (f < 0) item = __ldcg(R.refused + ref0 + k);
         const int inst = I.ninst > 1 ? csr_find(I.pofs, I.ninst + 1, gmoves[item].x) : 0;
         if (pending <= I.few_left) R.left[i] = item;
         else next[item] = atomicExch(head + partition_of(I, inst, bits, old_xy[item]), item);
@@ -487,7 +489,8 @@ __global__ void k_build_rest(Rounds R, int b, RoundBuild B, const int *refused, 
     const int nlost = __ldcg(R.lostcnt + b), head = __ldcg(R.head + b), n = nlost + B.total - head;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n + nref; i += gridDim.x * blockDim.x)
         R.left[atomicAdd(R.left_count, 1)] =
-            i < nlost ? __ldcg(R.lost[b & 1] + i) : (i < n ? __ldg(B.queue + head + i - nlost) : __ldcg(refused + i - n));
+            i < nlost ? __ldcg(R.lost[b & 1] + i)
+                      : (i < n ? __ldg(B.queue + head + i - nlost) : __ldcg(refused + i - n));
 }
 
 // Insertions by one warp each: the staged Bowyer-Watson insertion, else split and flips, with

@@ -157,7 +157,7 @@ __host__ __device__ constexpr unsigned tc_off(int r, int k, int K)
 
 // ---------------------------------------------------------------- the network
 
-constexpr int TC_M = 128;        // rows per tile = TMEM lanes = threads
+constexpr int TC_M = 128;        // rows per tile = TMEM lanes
 constexpr int TC_N3 = 32;        // the 18 outputs padded to a multiple of 16 (N of layer 3)
 constexpr unsigned TC_COLS = 128;  // TMEM columns: layer 1 at 0-63, layer 2 at 64-127, layer 3 at 0-31
 // shared-memory layout (bytes from a 1024-aligned base)
@@ -188,7 +188,8 @@ __device__ __forceinline__ void tc_stage_weights(unsigned char *tile, const unsi
         const int ch = tid + i * THREADS;
         c[i] = make_uint4(0, 0, 0, 0);
         if (ch < CHUNKS && ch / (K / 8) < live)
-            c[i] = make_uint4(__ldg(s32 + 4 * ch), __ldg(s32 + 4 * ch + 1), __ldg(s32 + 4 * ch + 2), __ldg(s32 + 4 * ch + 3));
+            c[i] = make_uint4(__ldg(s32 + 4 * ch), __ldg(s32 + 4 * ch + 1), __ldg(s32 + 4 * ch + 2),
+                              __ldg(s32 + 4 * ch + 3));
     }
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
@@ -469,8 +470,8 @@ __device__ __forceinline__ void tc_rows(unsigned d, unsigned ahi, unsigned amid,
 // at column c0 of the K-column tiles at hiofs / midofs, lo at column c0 - lo0 of the
 // 64-column lo tile.
 template <int H>
-__device__ __forceinline__ void tc_put3(unsigned char *S, unsigned hiofs, unsigned midofs, int r, int c0, int K, int lo0,
-                                        const float *v)
+__device__ __forceinline__ void tc_put3(unsigned char *S, unsigned hiofs, unsigned midofs, int r, int c0, int K,
+                                        int lo0, const float *v)
 {
 #pragma unroll
     for (int h = 0; h < H; ++h) {

@@ -139,3 +139,15 @@ def test_boxes_of_uneven_instances(n):
     bad[-1][-1] = (1 << 20, 5)
     with pytest.raises(kdt.KDTError):
         t.build_batch(bad)
+
+
+def test_points_left_out_in_a_batch():
+    """Instances that leave points out of the rounds beside some that do not."""
+    sets = [_rows(2000, 20, 26), W.uniform_points(3000, 26, 1), _rows(900, 30, 26), W.uniform_points(5, 26, 2),
+            _rows(1500, 10, 26), W.uniform_points(20000, 26, 3)]
+    t = _tri(domain_bits=26)
+    for _ in range(3):
+        t.build_batch(sets)
+        assert t.verify() == 0
+        for i, xy in enumerate(sets):
+            assert_same(t.export_triangles_inst(i), xy, "instance %d" % i)
