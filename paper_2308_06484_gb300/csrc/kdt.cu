@@ -175,7 +175,7 @@ struct kdt {
     int tune_count = 0;
     double tune_ms[9] = {0};
     // host side
-    int *hscal = nullptr;  // pinned copy of the scalars (and four words more)
+    int *hscal = nullptr;  // pinned copy of the scalars (and six words more)
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr, ev3 = nullptr;
     kdt_stats stats{};
     // learned locate proposal and its training rows (kdt_mlp.cuh)
@@ -441,19 +441,15 @@ int certify_and_repair(kdt *h, bool full, int s0, int nslots, int wraps, int *de
     return 0;
 }
 
-// the counters of `rounds` rounds in one buffer: heads, offsets and losers (rounds + 1
-// entries each), the lengths of the left and the refused list, the moves pending; `ops`
-// operations a round
-size_t round_counter_ints(int rounds) { return 3 * (size_t)(rounds + 1) + 3; }
+// the counters of `rounds` rounds in one buffer: the rounds' entries, the lengths of the left
+// and a build's refused list, the moves pending; `ops` operations a round
+size_t round_counter_ints(int rounds) { return 4 * (size_t)(rounds + 1) + 3; }
 
 Rounds make_rounds(const Buf &cnt, int rounds, const Buf &lost, const Buf &hdr, const Buf &rec, int ops)
 {
     Rounds R;
-    int *c = (int *)cnt.p;
-    R.head = c;
-    R.off = c + (rounds + 1);
-    R.lostcnt = c + 2 * (rounds + 1);
-    R.left_count = c + 3 * (rounds + 1);
+    R.cnt = (int4 *)cnt.p;
+    R.left_count = (int *)(R.cnt + rounds + 1);
     R.refused_count = R.left_count + 1;
     R.pending = R.left_count + 2;
     R.lost[0] = (int *)lost.p;
@@ -592,7 +588,7 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
     }
     const RoundMoves M{nullptr};
     auto left_warps = [ni](long long in) { return std::max<long long>(ni, in / LEFT_POINTS); };
-    int *hs = h->hscal + S_NUM;  // pinned: head, losers, left and refused so far
+    int *hs = h->hscal + S_NUM;  // pinned: a round's counters, the lengths of the left and the refused list
     int b = 0, pend = B.total, nlost = 0, nleft = 0, nref = 0, left_done = 0, ref_done = 0;
     long long in = R.base;  // points in, those left or refused among them
     while (b < ROUND_MAX && (pend > 0 || nref > ref_done)) {
@@ -625,14 +621,13 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
         }
         h->stats.kernel_launches += 2 * k;
         CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(hs, R.head + b, sizeof(int), cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(hs + 1, R.lostcnt + b, sizeof(int), cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(hs + 2, R.left_count, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(hs, R.cnt + b, sizeof(int4), cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(hs + 4, R.left_count, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
         if (sync_scalars(h)) return KDT_ERR_CUDA;
         if (h->hscal[S_STATUS]) return dev_to_abi(h->hscal[S_STATUS]);
         nlost = hs[1];
-        nleft = hs[2];
-        nref = hs[3];
+        nleft = hs[4];
+        nref = hs[5];
         pend = B.total - hs[0] + nlost;
         in = R.base + hs[0] - nlost;
     }
@@ -1224,6 +1219,7 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
         R.left = (int *)h->rm_left.p;
         R.refused = (int *)h->rm_ref.p;
         R.wide = R.refused;
+        R.refused_count = (int *)(R.cnt + nrounds - 1) + 2;
         I.pending = R.pending;
         I.left = R.left;
         I.few_left = std::min(FEW_LEFT, h->mcap / 4);  // (each can be left for later DQ_PASSES times)
@@ -1838,7 +1834,7 @@ int kdt_create(kdt **out, const kdt_config *cfg, int device, void *cuda_stream)
     h->cfg = c;
     if (cudaMalloc(&h->scal, S_NUM * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&h->counters, C_SLOTS * sizeof(unsigned long long)) != cudaSuccess ||
-        cudaMallocHost(&h->hscal, (S_NUM + 4) * sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&h->hscal, (S_NUM + 6) * sizeof(int)) != cudaSuccess ||
 
         cudaStreamCreateWithFlags(&h->cstream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreate(&h->ev0) != cudaSuccess || cudaEventCreate(&h->ev1) != cudaSuccess ||

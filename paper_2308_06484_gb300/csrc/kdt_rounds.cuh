@@ -54,13 +54,13 @@ constexpr int ROUND_BLOCKS = 16;            // ... its blocks per SM: 64 registe
                                             // 16 1.55, 20 1.75 ms a step
 constexpr int ROUND_LANES = 8;              // lanes of k_round_commit per operation
 
-// What one round works on: the losers of the round before (lost[b & 1], lostcnt[b] of
-// them), then fresh items from position head[b] of the queue.  Counters have one entry per
-// round, written by the round before, so a round's kernels read constants.
+// What one round works on: the losers of the round before (lost[b & 1]), then fresh items
+// of the queue.  Counters have one entry per round, written by the rounds before, so a
+// round's kernels read constants: one 16-byte load a thread, for every warp of the GPU reads
+// the same words (a word more cost 4 us in each kernel of thousands of blocks).
 struct Rounds {
-    int *head;      // [rounds + 1] next fresh item
-    int *off;       // [rounds + 1] operations planned before the round
-    int *lostcnt;   // [rounds + 1]
+    int4 *cnt;      // [rounds + 1] next fresh item, losers of the round before, refused items (in a
+                    // step's last round), operations planned before the round
     int *lost[2];   // item ids
     int4 *hdr;      // per operation of the round: item, triangles (0: plan again, -1: left to the
                     // other path), priority, k | ncav << 8 | edge << 24 | ghost << 25 | prop << 26
@@ -80,20 +80,27 @@ struct Rounds {
     int ops;        // room for operations of one round
 };
 
-// items of the refused list that a round with nwide < 0 takes after its nlost losers
-__device__ __forceinline__ int round_all_refused(const Rounds &R, int nlost)
+// items of the refused list that a round with nwide < 0 and counters c takes after its losers
+__device__ __forceinline__ int round_all_refused(const Rounds &R, const int4 &c)
 {
-    return min(__ldcg(R.refused_count), max(0, R.ops - nlost));
+    return min(c.z, max(0, R.ops - c.y));
+}
+
+__device__ __forceinline__ int *round_word(const Rounds &R, int b, int i)
+{
+    return reinterpret_cast<int *>(R.cnt + b) + i;
 }
 
 // the round's operations: losers, nw items of the wide list, fresh items from `head` (total:
 // length of the queue)
 __device__ __forceinline__ void round_window(const Rounds &R, int b, int total, int &nlost, int &nw, int &head,
-                                             int &count)
+                                             int &count, int &off)
 {
-    nlost = __ldcg(R.lostcnt + b);
-    head = __ldcg(R.head + b);
-    nw = R.nwide >= 0 ? R.nwide : round_all_refused(R, nlost);
+    const int4 c = __ldcg(R.cnt + b);
+    head = c.x;
+    nlost = c.y;
+    off = c.w;
+    nw = R.nwide >= 0 ? R.nwide : round_all_refused(R, c);
     int lim = R.ops;
     if (R.div > 0) {
         const int in = R.base + head - nlost;
@@ -168,12 +175,11 @@ __device__ __forceinline__ void round_plan(const Dev &d, const Rounds &R, int b,
                                            int nthreads)
 {
     constexpr bool MOVE = MODE != REGION_INSERT;
-    int nlost, nw, head, count;  // (nw > 0 in rounds of 32 lanes only)
-    round_window(R, b, total, nlost, nw, head, count);
-    const int off = __ldcg(R.off + b);
+    int nlost, nw, head, count, off;  // (nw > 0 in rounds of 32 lanes only)
+    round_window(R, b, total, nlost, nw, head, count, off);
     if (tid == 0) {
-        R.head[b + 1] = head + count - nlost - nw;
-        R.off[b + 1] = off + count;
+        *round_word(R, b + 1, 0) = head + count - nlost - nw;
+        *round_word(R, b + 1, 3) = off + count;
     }
     constexpr int PER_WARP = 32 / RL;
     const int l = threadIdx.x & (RL - 1), g0 = threadIdx.x & 31 & ~(RL - 1);
@@ -276,8 +282,8 @@ template <bool MOVE>
 __device__ __forceinline__ void round_commit(const Dev &d, const Rounds &R, int b, const RoundMoves &M, int total,
                                              int *sum, int tid, int nthreads)
 {
-    int nlost, nw, head, count;
-    round_window(R, b, total, nlost, nw, head, count);
+    int nlost, nw, head, count, off;
+    round_window(R, b, total, nlost, nw, head, count, off);
     const int lane = threadIdx.x & (ROUND_LANES - 1);
     const unsigned gm = 0xffu << (threadIdx.x & 24);  // this operation's lanes
     int nwin = 0, nlose = 0, degs = 0, flips = 0, edges = 0, ghosts = 0, props = 0, hits = 0;
@@ -335,7 +341,7 @@ __device__ __forceinline__ void round_commit(const Dev &d, const Rounds &R, int 
                 hits += (h.w >> 27) & 1;
             } else {
                 ++nlose;
-                R.lost[(b + 1) & 1][atomicAdd(R.lostcnt + b + 1, 1)] = h.x;
+                R.lost[(b + 1) & 1][atomicAdd(round_word(R, b + 1, 1), 1)] = h.x;
             }
         }
     }
@@ -377,7 +383,8 @@ __device__ __forceinline__ void round_clear(const Dev &d, const Rounds &R, int r
                                             const int3 *gmoves, const int2 *old_xy, int *head, int *next, int tid,
                                             int nthreads)
 {
-    const long long words = (long long)__ldcg(R.off + rounds) * RT;
+    const int4 end = __ldcg(R.cnt + rounds), last = __ldcg(R.cnt + rounds - 1);
+    const long long words = (long long)end.w * RT;
     for (long long i = 4ll * tid; i < words; i += 4ll * nthreads) {
         const int4 s = __ldcg(reinterpret_cast<const int4 *>(R.slots + i));
         if (s.x >= 0) d.tn[s.x].w = 0;
@@ -385,8 +392,8 @@ __device__ __forceinline__ void round_clear(const Dev &d, const Rounds &R, int r
         if (s.z >= 0) d.tn[s.z].w = 0;
         if (s.w >= 0) d.tn[s.w].w = 0;
     }
-    const int nleft = __ldcg(R.left_count), nlost = __ldcg(R.lostcnt + rounds), fresh = __ldcg(R.head + rounds);
-    const int ref0 = round_all_refused(R, __ldcg(R.lostcnt + rounds - 1)), nref = __ldcg(R.refused_count) - ref0;
+    const int nleft = __ldcg(R.left_count), nlost = end.y, fresh = end.x;
+    const int ref0 = round_all_refused(R, last), nref = last.z - ref0;
     const int pending = nleft + nlost + nref + m - fresh;
     if (tid == 0) *R.pending = pending;
     for (int i = tid; i < pending; i += nthreads) {
@@ -455,7 +462,8 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_step_small(Dev d, const int3 
         round_commit<true>(d, R, b, M, m, sum, tid, SMALL_THREADS);
         phase();
         ++b;
-        const int now = __ldcg(R.lostcnt + b) + m - __ldcg(R.head + b);
+        const int4 c = __ldcg(R.cnt + b);
+        const int now = c.y + m - c.x;
         if (now == 0 || now == pending) break;
         pending = now;
     }
@@ -486,7 +494,8 @@ __global__ void k_build_queue(RoundBuild B, const int *lvoff, int level, int ite
 // warp-wide path
 __global__ void k_build_rest(Rounds R, int b, RoundBuild B, const int *refused, int nref)
 {
-    const int nlost = __ldcg(R.lostcnt + b), head = __ldcg(R.head + b), n = nlost + B.total - head;
+    const int4 c = __ldcg(R.cnt + b);
+    const int nlost = c.y, head = c.x, n = nlost + B.total - head;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n + nref; i += gridDim.x * blockDim.x)
         R.left[atomicAdd(R.left_count, 1)] =
             i < nlost ? __ldcg(R.lost[b & 1] + i)
