@@ -490,16 +490,19 @@ void launch_round(kdt *h, cudaStream_t st, const Dev &d, const Rounds &R, int b,
 // large ones their attempts.  1e6 points: 4 / 0 20.4 ms, 8 / 0 10.8, 12 / 0 9.8, 12 / 2048 9.7,
 // 12 / 8192 11.5, 16 / 4096 9.9 against 10.3 with 12 / 4096.
 constexpr int BUILD_DIV = 12, BUILD_FEW = 2048;
-// At least so many rounds between two looks at the counters.  What the rounds left out is
-// inserted there, while its cavities are as small as they will be: a dense row of 10,000
-// points facing 100 (degrees of 100 and more) took 2.6 s with all of it at the end, 50 ms so
-// (60-440 with one warp per insertion throughout); on a lattice of 300 x 300, one build in
-// ten left so many neighbouring points that their insertions ran out of retries.
+// At least so many rounds between two looks at the counters, and at most as many new points as
+// are in.  What the rounds left out is inserted there, while its cavities are as small as
+// they will be (and the hull edges a point outside the hull sees as few: the insertion takes
+// 60): a dense row of 10,000 points facing 100 (degrees of 100 and more) took 2.6 s with all
+// of it at the end, 45 ms with four times the points between two looks, 27 ms so (46-440
+// with one warp per insertion throughout); on a lattice of 300 x 300, one build in ten left
+// so many neighbouring points that their insertions ran out of retries.
 constexpr int BUILD_ROUNDS = 8;
 // Points in per warp that inserts what was left out: the cavities have more than 32 triangles,
 // and warps that meet lose their claims and leave edges to repair; fewer warps wait for one
 // another.  The rows 55 ms / 52 / 60 / 105, 3,000 rings of 60 points with a centre each 7.2 /
-// 6.8 / 8.5 / 800, with 64 / 128 / 512 / all points a warp.
+// 6.8 / 8.5 / 800, with 64 / 128 / 512 / all points a warp (four times the points between
+// two looks).
 constexpr int LEFT_POINTS = 128;
 
 // One warp per insertion (k_insert_warps), at most `most` of them at once.
@@ -589,9 +592,13 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
     const RoundMoves M{nullptr};
     auto left_warps = [ni](long long in) { return std::max<long long>(ni, in / LEFT_POINTS); };
     int *hs = h->hscal + S_NUM;  // pinned: a round's counters, the lengths of the left and the refused list
-    int b = 0, pend = B.total, nlost = 0, nleft = 0, nref = 0, left_done = 0, ref_done = 0;
+    int b = 0, pend = B.total, head = 0, nlost = 0, nleft = 0, nref = 0, left_done = 0, ref_done = 0;
     long long in = R.base;  // points in, those left or refused among them
     while (b < ROUND_MAX && (pend > 0 || nref > ref_done)) {
+        // (the points in double at most before what is left out is looked at)
+        RoundBuild S = B;
+        S.total = (int)std::min<long long>(B.total, head + std::max(64ll, in));
+        long long todo = nlost + S.total - head;
         if (nleft > left_done) {
             k_clear_owner<<<thread_grid(h, nslots, 256), 256, 0, st>>>(d.tn, s0, nslots);
             launch_insert_warps(h, d, R.left + left_done, nleft - left_done, left_warps(in), B, 0, nullptr);
@@ -606,17 +613,17 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
         if (nref > ref_done && (pend == 0 || nref - ref_done >= std::max<long long>(8, in / 1024))) {
             R.wide = R.refused + ref_done;
             R.nwide = std::min(nref - ref_done, ops - nlost);
-            launch_round<REGION_INSERT>(h, st, d, R, b++, nlost + R.nwide, M, B, true, true);
+            launch_round<REGION_INSERT>(h, st, d, R, b++, nlost + R.nwide, M, S, true, true);
             ref_done += R.nwide;
-            pend += R.nwide;
+            todo += R.nwide;
             R.nwide = 0;
             ++k;
         }
-        // rounds until the points in have grown fourfold, if every operation won
-        for (long long est = in; b < ROUND_MAX && (k < BUILD_ROUNDS || (est < 4 * in && est < np)); ++b, ++k) {
-            const long long most = std::min<long long>({(long long)ops, (long long)pend, window(est)});
+        // rounds until the points in have doubled, if every operation won
+        for (long long est = in; b < ROUND_MAX && (k < BUILD_ROUNDS || (est < 2 * in && est < np)); ++b, ++k) {
+            const long long most = std::min<long long>({(long long)ops, todo, window(est)});
             const bool wide = 32 * most <= (long long)ROUND_THREADS * 32 * sm_count(h->device);
-            launch_round<REGION_INSERT>(h, st, d, R, b, most, M, B, wide, wide);
+            launch_round<REGION_INSERT>(h, st, d, R, b, most, M, S, wide, wide);
             est = std::min(est + most, np);
         }
         h->stats.kernel_launches += 2 * k;
@@ -625,11 +632,12 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
         CK(cudaMemcpyAsync(hs + 4, R.left_count, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
         if (sync_scalars(h)) return KDT_ERR_CUDA;
         if (h->hscal[S_STATUS]) return dev_to_abi(h->hscal[S_STATUS]);
+        head = hs[0];
         nlost = hs[1];
         nleft = hs[4];
         nref = hs[5];
-        pend = B.total - hs[0] + nlost;
-        in = R.base + hs[0] - nlost;
+        pend = B.total - head + nlost;
+        in = R.base + head - nlost;
     }
     k_clear_owner<<<thread_grid(h, nslots, 256), 256, 0, st>>>(d.tn, s0, nslots);
     h->stats.kernel_launches++;
