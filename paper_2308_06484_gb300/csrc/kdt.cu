@@ -388,8 +388,8 @@ int kinetic_blocks(kdt *h)
     return sm_count(h->device) * per_sm;
 }
 
-// Certify slots [s0, s0 + nslots) (or the dirty list when !full), then repair until
-// no violation is left.  A full pass must see `wraps` hull windings (one per
+// Certify slots [s0, s0 + nslots) (or the dirty list when !full, while it holds all that was
+// written), then repair until no violation is left.  A full pass must see `wraps` hull windings (one per
 // instance in the range) and, when the range is `whole` (not during a build), a triangle
 // in every slot.  Returns a CUDA/ABI error; the device status goes to
 // *dev_status.
@@ -414,6 +414,10 @@ int certify_and_repair(kdt *h, bool full, int s0, int nslots, int wraps, int *de
         if (sync_scalars(h)) return KDT_ERR_CUDA;
         *dev_status = h->hscal[S_STATUS];
         if (*dev_status) return 0;
+        if (!full && h->hscal[S_DIRTY] > h->dirty_cap) {
+            full = true;
+            continue;
+        }
         int nv = h->hscal[S_VIOL];
         h->stats.violations += nv;
         if (nv == 0) {
@@ -430,12 +434,6 @@ int certify_and_repair(kdt *h, bool full, int s0, int nslots, int wraps, int *de
         if (sync_scalars(h)) return KDT_ERR_CUDA;
         *dev_status = h->hscal[S_STATUS];
         if (*dev_status) return 0;
-        if (!full && h->hscal[S_DIRTY] > h->dirty_cap) {
-            full = true;
-            s0 = 0;
-            nslots = h->cap;
-            wraps = h->ninst;
-        }
     }
     *dev_status = DEV_INTERNAL;
     return 0;
@@ -504,6 +502,18 @@ constexpr int BUILD_ROUNDS = 8;
 // 6.8 / 8.5 / 800, with 64 / 128 / 512 / all points a warp (four times the points between
 // two looks).
 constexpr int LEFT_POINTS = 128;
+constexpr int BUILD_DIRTY = 1 << 18;  // triangles these insertions write at a time, at least
+
+// The list of slots written outside the staged paths: room for cap of them.
+int ensure_dirty(kdt *h, int cap)
+{
+    if (cap <= h->dirty_cap) return 0;
+    h->dirty_cap = 0;
+    h->gen++;  // a captured step graph holds the old pointer
+    if (dalloc(&h->dirty, (size_t)cap)) return KDT_ERR_CUDA;
+    h->dirty_cap = cap;
+    return 0;
+}
 
 // One warp per insertion (k_insert_warps), at most `most` of them at once.
 void launch_insert_warps(kdt *h, const Dev &d, const int *left, int items, long long most, const RoundBuild &B,
@@ -601,11 +611,18 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
         long long todo = nlost + S.total - head;
         if (nleft > left_done) {
             k_clear_owner<<<thread_grid(h, nslots, 256), 256, 0, st>>>(d.tn, s0, nslots);
-            launch_insert_warps(h, d, R.left + left_done, nleft - left_done, left_warps(in), B, 0, nullptr);
+            // (the rounds' plans need every edge locally Delaunay: what the insertions wrote is
+            // certified; every slot would be 5 ms on 16e6 points)
+            if (ensure_dirty(h, BUILD_DIRTY)) return KDT_ERR_CUDA;
+            Dev dw = d;
+            dw.dirty = h->dirty;
+            dw.dirty_cap = h->dirty_cap;
+            CK(cudaMemsetAsync(h->scal + S_DIRTY, 0, sizeof(int), st));
+            launch_insert_warps(h, dw, R.left + left_done, nleft - left_done, left_warps(in), B, 0, nullptr);
             h->stats.kernel_launches++;
             CK(cudaGetLastError());
-            int ds = 0;  // (the rounds' plans need every edge locally Delaunay)
-            if (certify_and_repair(h, true, s0, nslots, ni, &ds, false)) return KDT_ERR_CUDA;
+            int ds = 0;
+            if (certify_and_repair(h, false, s0, nslots, ni, &ds, false)) return KDT_ERR_CUDA;
             if (ds) return dev_to_abi(ds);
             left_done = nleft;
         }
@@ -847,8 +864,7 @@ int ensure_moves(kdt *h, int64_t m)
     h->mcap = c;
     long long dc = 64ll * c + 4096;
     if (dc > (1ll << 30)) dc = 1ll << 30;
-    if (dalloc(&h->dirty, (size_t)dc)) return KDT_ERR_CUDA;
-    h->dirty_cap = (int)dc;
+    if (ensure_dirty(h, (int)dc)) return KDT_ERR_CUDA;
     h->gen++;
     return 0;
 }
