@@ -81,16 +81,23 @@ typedef struct {
     int32_t timing;        /* 1: time the rounds of moves and the kinetic kernel with CUDA
                               events (kdt_stats)                                            */
     int32_t warps_per_block; /* kinetic kernel launch shape (default 4)                      */
-    int32_t build_warps;   /* warps inserting concurrently during a build (0 = auto)         */
-    int32_t kinetic_warps; /* warps moving points concurrently in a step (0 = one per cell)  */
+    int32_t build_warps;   /* > 0: a build inserts with so many warps at once, a warp per
+                              point, level by level, instead of in rounds (0)                */
+    int32_t kinetic_warps; /* > 0: so many warps do all of a step's moves, instead of rounds
+                              first (0; then one warp per cell does what the rounds leave)   */
     int32_t debug;         /* bit 0: on an in-step failure keep the failed state (no
                               fallback, no roll-back) so kdt_export_store can inspect it;
                               bit 1: record the kinetic launch's timeline (span_* stats)     */
     int32_t use_graph;     /* 1: launch each step as one captured CUDA graph (default)       */
     int32_t points_per_partition; /* partition size of batched instances (0 = 256)           */
-    int32_t warps_per_partition;  /* warps sharing one partition's moves (0 = 1)             */
+    int32_t warps_per_partition;  /* warps sharing one partition's moves (0 = 1).  This, the
+                              order of the partitions and bit 0 of plan say how the kinetic
+                              kernel takes moves: all of a step that does not go through
+                              rounds (a variant, training rows, a proposal inside the move,
+                              kinetic_warps), else the few that the rounds leave              */
     int32_t autotune;      /* 1: time the first steps over points per partition {128, 256,
-                              512} x warps per partition {1, 2, 4} and keep the fastest       */
+                              512} x warps per partition {1, 2, 4} and keep the fastest (steps
+                              in rounds differ by little more than their spread)              */
     int32_t variant;       /* 0: every move deletes and re-inserts the point (the paper's
                               method, default).  1: first test whether the point can move
                               in place: every triangle of its star stays counter-clockwise

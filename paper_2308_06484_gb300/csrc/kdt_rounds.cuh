@@ -25,16 +25,17 @@
 // per move or insertion, claiming star and ring by compare-and-swap, re-reading them under
 // the claims and certifying afterwards took about 6,500 warp instructions an operation
 // in code too large for the instruction caches ("no instruction" 10-15 stalled cycles per
-// issue).  Planned without claims by 16 lanes an operation takes about 850.
-//   step, 1e6 uniform points, 4096 moves          125 -> 85 us
-//   step, 16e6 clustered points, 140,000 moves   2.75 -> 1.5 ms
+// issue).  The plan takes 1,970 with a warp to itself (12 of 32 lanes active), 1,460 where two
+// share a warp.
+//   step, 1e6 uniform points, 4096 moves          125 -> 77 us
+//   step, 16e6 clustered points, 140,000 moves   2.75 -> 1.25 ms (median)
 //   step, 512 instances, 212,000 moves            2.6 -> 0.8 ms
 //   step, 2e5 points, 1,950 moves that leave their star   390 -> 180 us
-//   rebuild, 1e6 uniform points                  28.8 -> 10.5 ms
-//   rebuild, 128 instances, 1.5e6 points         37   -> 9.8 ms
-// Bound now: the latency of the plan's chain (12-27 us a round of a few thousand operations)
-// times the number of rounds; with 1e5 operations or more, the SMs' issue slots (41 %
-// busy) and the spread of the loads over L2.
+//   rebuild, 1e6 uniform points                  28.8 -> 9.6 ms
+//   rebuild, 128 instances, 1.5e6 points         37   -> 9.6 ms
+// Bound now: the latency of the plan's chain (12-27 us a round of a few thousand operations,
+// 42 % of the issue slots used) times the number of rounds; with 1e5 operations or more,
+// the issue slots and the spread of the loads over L2.
 //
 // Owner words keep the claims of earlier rounds until the end (a priority starts with
 // the round's number, so older ones always lose); only k_round_clear or k_clear_owner
