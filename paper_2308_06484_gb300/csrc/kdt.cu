@@ -128,8 +128,8 @@ struct kdt {
     Buf key, bord, hist, hoff, exp_cnt, exp_off, exp_fill, exp_out, exp_rows;
     Buf btab, blev;  // batched build: per-instance tables, per-level item offsets
     // rounds (kdt_rounds.cuh): of a build, and of the steps
-    Buf rb_cnt, rb_lost, rb_hdr, rb_rec, rb_queue, rb_left, rb_ref;
-    Buf rm_cnt, rm_lost, rm_hdr, rm_rec, rm_slots, rm_left, rm_ref;
+    Buf rb_cnt, rb_lost, rb_hdr, rb_rec, rb_queue, rb_left;
+    Buf rm_cnt, rm_lost, rm_hdr, rm_rec, rm_slots, rm_left;
     int rm_cap = 0, rm_ops = 0;  // moves of a step, operations of a round they have room for
     int rm_layout = 0;           // rounds the counters have room for (a small step's too)
     // d-calculation: results, running minimum (per N)
@@ -575,12 +575,11 @@ int insert_rounds(kdt *h, Dev d, RoundBuild B, const std::vector<int> &lv, const
     if (grow(h->rb_cnt, round_counter_ints(ROUND_MAX) * sizeof(int)) ||
         grow(h->rb_lost, 2 * (size_t)ops * sizeof(int)) || grow(h->rb_hdr, (size_t)ops * sizeof(int4)) ||
         grow(h->rb_rec, (size_t)ops * 2 * RT * sizeof(int4)) ||
-        grow(h->rb_queue, (size_t)np * sizeof(int)) || grow(h->rb_left, (size_t)np * sizeof(int)) ||
-        grow(h->rb_ref, (size_t)np * sizeof(int)))
+        grow(h->rb_queue, (size_t)np * sizeof(int)) || grow(h->rb_left, 2 * (size_t)np * sizeof(int)))
         return KDT_ERR_CUDA;
     Rounds R = make_rounds(h->rb_cnt, ROUND_MAX, h->rb_lost, h->rb_hdr, h->rb_rec, ops);
     R.left = (int *)h->rb_left.p;
-    R.refused = (int *)h->rb_ref.p;
+    R.refused = R.left + np;
     R.div = BUILD_DIV;
     R.few = BUILD_FEW;
     R.base = 3 * ni;
@@ -880,16 +879,18 @@ bool step_in_rounds(const kdt *h)
            h->cfg.kinetic_warps == 0;
 }
 
-// Room for the rounds of a step of m moves.
+// Room for the rounds of a step of m <= mcap moves, and of others of its class as far as the
+// move list's own buffers go (a little more room at every step would be a capture at every
+// step).
 int ensure_rounds(kdt *h, int64_t m)
 {
     if (m <= h->rm_cap) return 0;
-    const int cap = (int)std::max<int64_t>(m, 1024), ops = std::min(cap, ROUND_OPS);
+    const int cap = (int)std::min<long long>(h->mcap, class_moves(step_class(m))), ops = std::min(cap, ROUND_OPS);
     const int rounds = class_rounds(step_class(cap)), layout = std::max(rounds, SMALL_ROUNDS);
     if (grow(h->rm_cnt, round_counter_ints(layout) * sizeof(int)) || grow(h->rm_lost, 2 * (size_t)ops * sizeof(int)) ||
         grow(h->rm_hdr, (size_t)ops * sizeof(int4)) || grow(h->rm_rec, (size_t)ops * 2 * RT * sizeof(int4)) ||
         grow(h->rm_slots, std::max((size_t)rounds * ops, (size_t)SMALL_ROUNDS * SMALL_MOVES) * RT * sizeof(int)) ||
-        grow(h->rm_left, (size_t)cap * sizeof(int)) || grow(h->rm_ref, (size_t)cap * sizeof(int)))
+        grow(h->rm_left, 2 * (size_t)cap * sizeof(int)))
         return KDT_ERR_CUDA;
     h->rm_ops = ops;
     h->rm_cap = cap;
@@ -1019,8 +1020,8 @@ void free_state(kdt *h)
     h->mcap = 0; h->dirty_cap = 0; h->scan_tmp_cap = 0; h->rm_cap = 0;
     Buf *bs[] = {&h->key, &h->bord, &h->hist, &h->hoff, &h->exp_cnt, &h->exp_off, &h->exp_fill, &h->exp_out,
                  &h->exp_rows, &h->btab, &h->blev,
-                 &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left, &h->rb_ref,
-                 &h->rm_cnt, &h->rm_lost, &h->rm_hdr, &h->rm_rec, &h->rm_slots, &h->rm_left, &h->rm_ref,
+                 &h->rb_cnt, &h->rb_lost, &h->rb_hdr, &h->rb_rec, &h->rb_queue, &h->rb_left,
+                 &h->rm_cnt, &h->rm_lost, &h->rm_hdr, &h->rm_rec, &h->rm_slots, &h->rm_left,
                  &h->dc_dist, &h->dc_cmin, &h->dc_scal};
     for (Buf *b : bs) free_buf(*b);
 }
@@ -1241,7 +1242,7 @@ int enqueue_step(kdt *h, cudaStream_t st, const Dev &d, const int3 *mp, int mi, 
         R = make_rounds(h->rm_cnt, h->rm_layout, h->rm_lost, h->rm_hdr, h->rm_rec, h->rm_ops);
         R.slots = (int *)h->rm_slots.p;
         R.left = (int *)h->rm_left.p;
-        R.refused = (int *)h->rm_ref.p;
+        R.refused = R.left + h->rm_cap;
         R.wide = R.refused;
         R.refused_count = (int *)(R.cnt + nrounds - 1) + 2;
         I.pending = R.pending;
