@@ -68,18 +68,15 @@ def bytes_per_update(k_old, k_new):
 
 BYTES_K6 = bytes_per_update(6, 6)
 
-# DRAM bytes (read + write) per moved point of one k_kinetic launch, from ncu's
-# dram__bytes_read.sum + dram__bytes_write.sum (profiles/), valid only for the kernel
-# sources it was taken on (their SHA-256 prefix) and the workload it was taken on; the
-# bench line reports it scaled to the launch's moves, null otherwise.
+# DRAM bytes (read + write) per moved point of one step's rounds and k_kinetic, from ncu's
+# dram__bytes_read.sum + dram__bytes_write.sum over their launches (profiles/), valid only
+# for the kernel sources it was taken on (their SHA-256 prefix) and the workload it was
+# taken on; the bench line reports it scaled to the step's moves, null otherwise.
 KINETIC_TRAFFIC = {
-    # 16e6-point workload, 3 launches of 165,068 moves: 441.5, 440.9, 438.7 MB (the
-    # triangle store as 32-byte records)
-    "c3": {"sources": "505f12924c6ce36f", "bytes_per_move": 2668.0},
-    # 1e6-point workload, 2 launches of 4,096 moves: 15.64, 15.69 MB, taken with the
-    # two halves of a triangle in separate arrays (no capture of the current sources:
-    # the traffic is reported as null)
-    "c2": {"sources": "0a5e0b49bcda6ab7", "bytes_per_move": 3824.0},
+    # 16e6-point workload, 3 steps of 165,068 moves: 967.2, 966.0, 963.8 MB
+    "c3": {"sources": "262704249766158c", "bytes_per_move": 5850.3},
+    # 1e6-point workload, 3 steps of 4,096 moves: 15.86, 15.68, 15.73 MB
+    "c2": {"sources": "262704249766158c", "bytes_per_move": 3847.0},
 }
 
 
